@@ -38,15 +38,21 @@ __host__ __device__ __forceinline__ double2 conj2(double2 a) { return make_doubl
 __host__ __device__ __forceinline__ float2 conj2(float2 a) { return make_float2(a.x, -a.y); }
 // i * a
 template <typename T> __host__ __device__ __forceinline__ T mul_i(T a) { T r; r.x = -a.y; r.y = a.x; return r; }
-// acc += a * b
+// acc += a * b, one product at a time, so that each contracts into a fused
+// multiply-add on the accumulator: four instructions (the sum of both products
+// added at the end takes six, and the FP64 kernels are bound by that pipe)
 template <typename T> __host__ __device__ __forceinline__ void cfma(T &acc, T a, T b) {
-    acc.x += a.x * b.x - a.y * b.y;
-    acc.y += a.x * b.y + a.y * b.x;
+    acc.x += a.x * b.x;
+    acc.y += a.x * b.y;
+    acc.x -= a.y * b.y;
+    acc.y += a.y * b.x;
 }
 // acc += conj(a) * b
 template <typename T> __host__ __device__ __forceinline__ void cfmac(T &acc, T a, T b) {
-    acc.x += a.x * b.x + a.y * b.y;
-    acc.y += a.x * b.y - a.y * b.x;
+    acc.x += a.x * b.x;
+    acc.y += a.x * b.y;
+    acc.x += a.y * b.y;
+    acc.y -= a.y * b.x;
 }
 
 template <typename TO, typename TI> __host__ __device__ __forceinline__ TO cvt(TI a);
