@@ -76,8 +76,10 @@ __global__ void __launch_bounds__(RED_THREADS) dot_kernel(const TX *__restrict__
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         TX u = x[i];
         TY v = y[i];
-        ar += (A)u.x * (A)v.x + (A)u.y * (A)v.y;
-        ai += (A)u.x * (A)v.y - (A)u.y * (A)v.x;
+        ar += (A)u.x * (A)v.x;  // one product at a time: fused multiply-adds (the FP64 pipe bounds these loops)
+        ai += (A)u.x * (A)v.y;
+        ar += (A)u.y * (A)v.y;
+        ai -= (A)u.y * (A)v.x;
     }
     finish(make_double2((double)ar, (double)ai), part, count, out, true);
 }
@@ -89,7 +91,8 @@ __global__ void __launch_bounds__(RED_THREADS) norm2_kernel(const T *__restrict_
     A a = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         T u = x[i];
-        a += (A)u.x * (A)u.x + (A)u.y * (A)u.y;
+        a += (A)u.x * (A)u.x;
+        a += (A)u.y * (A)u.y;
     }
     finish(make_double2((double)a, 0.0), part, count, out, false);
 }
@@ -111,8 +114,10 @@ __global__ void __launch_bounds__(RED_THREADS) multidot_kernel(MultiDotArgs<T, K
 #pragma unroll
         for (int j = 0; j < K; ++j) {
             T u = a.v[j][i];
-            ar[j] += (A)u.x * (A)y.x + (A)u.y * (A)y.y;
-            ai[j] += (A)u.x * (A)y.y - (A)u.y * (A)y.x;
+            ar[j] += (A)u.x * (A)y.x;
+            ai[j] += (A)u.x * (A)y.y;
+            ar[j] += (A)u.y * (A)y.y;
+            ai[j] -= (A)u.y * (A)y.x;
         }
     }
     __shared__ double2 sh[32];

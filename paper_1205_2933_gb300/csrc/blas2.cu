@@ -18,8 +18,10 @@ __global__ void caxpy_kernel(T *__restrict__ y, double2 ad, const T *__restrict_
     const R ar = (R)ad.x, ai = (R)ad.y;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         T xv = x[i], yv = y[i];
-        yv.x += ar * xv.x - ai * xv.y;
-        yv.y += ar * xv.y + ai * xv.x;
+        yv.x += ar * xv.x;
+        yv.y += ar * xv.y;
+        yv.x -= ai * xv.y;
+        yv.y += ai * xv.x;
         y[i] = yv;
     }
 }
@@ -120,17 +122,21 @@ template <typename T>
 __global__ void multiaxpy_dev_kernel(T *__restrict__ w, MultiArgs<T> a, const double *__restrict__ s, int ibase,
                                      double sgn, int64_t n) {
     using R = typename Real<T>::type;
-    R cr[32], ci[32];
-    for (int j = 0; j < a.k; ++j) {
-        cr[j] = (R)(sgn * s[ibase + 2 * j]);
-        ci[j] = (R)(sgn * s[ibase + 2 * j + 1]);
+    __shared__ R cr[32], ci[32];  // (indexed registers would live in local memory)
+    if (threadIdx.x < a.k) {
+        cr[threadIdx.x] = (R)(sgn * s[ibase + 2 * threadIdx.x]);
+        ci[threadIdx.x] = (R)(sgn * s[ibase + 2 * threadIdx.x + 1]);
     }
+    __syncthreads();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         T v = w[i];
+#pragma unroll 8
         for (int j = 0; j < a.k; ++j) {
             T u = a.p[j][i];
-            v.x += cr[j] * u.x - ci[j] * u.y;
-            v.y += cr[j] * u.y + ci[j] * u.x;
+            v.x += cr[j] * u.x;
+            v.y += cr[j] * u.y;
+            v.x -= ci[j] * u.y;
+            v.y += ci[j] * u.x;
         }
         w[i] = v;
     }

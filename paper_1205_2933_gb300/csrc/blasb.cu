@@ -77,7 +77,8 @@ __global__ void __launch_bounds__(BT) norm2_b_kernel(const T *__restrict__ x, in
     A a = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         T u = x[i];
-        a += u.x * u.x + u.y * u.y;
+        a += u.x * u.x;
+        a += u.y * u.y;
     }
     double2 m[1] = {make_double2((double)a, 0.0)};
     finish_b<1, false>(m, part, count, s, base, stride);
@@ -101,8 +102,10 @@ __global__ void __launch_bounds__(BT) multidot_b_kernel(VArgs<T, K> va, const T 
 #pragma unroll
         for (int j = 0; j < K; ++j) {
             T u = va.v[j][off + i];
-            ar[j] += u.x * y.x + u.y * y.y;
-            ai[j] += u.x * y.y - u.y * y.x;
+            ar[j] += u.x * y.x;
+            ai[j] += u.x * y.y;
+            ar[j] += u.y * y.y;
+            ai[j] -= u.y * y.x;
         }
     }
     double2 m[K];
@@ -122,17 +125,21 @@ __global__ void multiaxpy_b_kernel(T *__restrict__ w, MArgs<T> a, const double *
     using R = typename RealB<T>::type;
     const int r = blockIdx.y;
     const size_t off = (size_t)r * n;
-    R cr[32], ci[32];
-    for (int j = 0; j < a.k; ++j) {
-        cr[j] = (R)(sgn * s[base + r * stride + 2 * j]);
-        ci[j] = (R)(sgn * s[base + r * stride + 2 * j + 1]);
+    __shared__ R cr[32], ci[32];  // (indexed registers would live in local memory)
+    if (threadIdx.x < a.k) {
+        cr[threadIdx.x] = (R)(sgn * s[base + r * stride + 2 * threadIdx.x]);
+        ci[threadIdx.x] = (R)(sgn * s[base + r * stride + 2 * threadIdx.x + 1]);
     }
+    __syncthreads();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         T v = w[off + i];
+#pragma unroll 8
         for (int j = 0; j < a.k; ++j) {
             T u = a.v[j][off + i];
-            v.x += cr[j] * u.x - ci[j] * u.y;
-            v.y += cr[j] * u.y + ci[j] * u.x;
+            v.x += cr[j] * u.x;
+            v.y += cr[j] * u.y;
+            v.x -= ci[j] * u.y;
+            v.y += ci[j] * u.x;
         }
         w[off + i] = v;
     }
@@ -239,6 +246,18 @@ __global__ void cg_pxd_b_kernel(T *__restrict__ x, T *pout, const T *__restrict_
     if (mode == 0 && blockIdx.x == 0 && threadIdx.x == 0) sr[ia + NP] = (double)a;
 }
 
+// out_r = x_r / |x_r| in FP64, |x_r|^2 in s[base + r*stride]
+template <typename T>
+__global__ void normalised_b_kernel(double2 *__restrict__ out, const T *__restrict__ x, const double *__restrict__ s,
+                                    int base, int stride, int64_t n) {
+    const size_t off = (size_t)blockIdx.y * n;
+    const double a = 1.0 / sqrt(s[base + blockIdx.y * stride]);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const T v = x[off + i];
+        out[off + i] = make_double2(a * (double)v.x, a * (double)v.y);
+    }
+}
+
 // w_r *= sc[r];  res_r -= al[r] * w_r   (GCR direction normalisation and residual update)
 template <typename T>
 __global__ void gcr_wr_b_kernel(T *__restrict__ w, T *__restrict__ res, const double *__restrict__ sc,
@@ -264,17 +283,21 @@ __global__ void combo_b_kernel(T *__restrict__ x, MArgs<T> a, const double2 *__r
     using R = typename RealB<T>::type;
     const int r = blockIdx.y;
     const size_t off = (size_t)r * n;
-    R cr[32], ci[32];
-    for (int j = 0; j < a.k; ++j) {
-        cr[j] = (R)g[r * a.k + j].x;
-        ci[j] = (R)g[r * a.k + j].y;
+    __shared__ R cr[32], ci[32];
+    if (threadIdx.x < a.k) {
+        cr[threadIdx.x] = (R)g[r * a.k + threadIdx.x].x;
+        ci[threadIdx.x] = (R)g[r * a.k + threadIdx.x].y;
     }
+    __syncthreads();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         T v = x[off + i];
+#pragma unroll 8
         for (int j = 0; j < a.k; ++j) {
             T u = a.v[j][off + i];
-            v.x += cr[j] * u.x - ci[j] * u.y;
-            v.y += cr[j] * u.y + ci[j] * u.x;
+            v.x += cr[j] * u.x;
+            v.y += cr[j] * u.y;
+            v.x -= ci[j] * u.y;
+            v.y += ci[j] * u.x;
         }
         x[off + i] = v;
     }
@@ -481,6 +504,13 @@ void cg_pxd_b(dwf_ctx *c, T *x, T *pout, const T *pin, T *const *pend, int np, c
 }
 
 template <typename T>
+void normalised_b(dwf_ctx *c, double2 *out, const T *x, int base, int stride, int64_t n, int nrhs) {
+    dim3 g = grid_b(c, n, nrhs, 16);
+    normalised_b_kernel<T><<<g, BT, 0, c->stream>>>(out, x, c->scal.as<double>(), base, stride, n);
+    DWF_CHECK_LAUNCH();
+}
+
+template <typename T>
 void gcr_wr_b(dwf_ctx *c, T *w, T *res, const double *sc, const double2 *al, int64_t n, int nrhs) {
     dim3 g = grid_b(c, n, nrhs, 16);
     gcr_wr_b_kernel<T><<<g, BT, 0, c->stream>>>(w, res, sc, al, n);
@@ -534,6 +564,7 @@ void cg_chunk_b(dwf_ctx *c, T *x, T *p, T *const *Z, int m, bool next, bool xini
     template void cg_combine_b<T>(dwf_ctx *, T *, T *const *, int, int, int, int, int, int64_t, int);        \
     template void cg_chunk_b<T>(dwf_ctx *, T *, T *, T *const *, int, bool, bool, int, int, int, int, int, int,   \
                                 int64_t, int);                                                                 \
+    template void normalised_b<T>(dwf_ctx *, double2 *, const T *, int, int, int64_t, int);                   \
     template void gcr_wr_b<T>(dwf_ctx *, T *, T *, const double *, const double2 *, int64_t, int);            \
     template void combo_b<T>(dwf_ctx *, T *, T *const *, int, const double2 *, int64_t, int);
 INSTB(float2)

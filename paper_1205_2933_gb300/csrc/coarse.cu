@@ -146,13 +146,12 @@ __device__ __forceinline__ void fine_face_hop(C<R> acc12[12], const C<R> *ql, co
     }
 }
 
-// F[xc][dd][k][l], dd = 2*mu + (dir < 0): block-face contributions of one hop.
-// FINE: hop = -1/2 (1 -+ g_mu) U q_l(x +- mu) with boundary sign (the fine D);
-// else: hop = Y_d(x) q_l(x +- mu) of the finer coarse level's stencil.
-template <int NV, bool FINE, typename R>
+// F[xc][dd][k][l], dd = 2*mu + (dir < 0): block-face contributions of one hop
+// Y_d(x) q_l(x +- mu) of a coarse level's stencil (the fine level stores its
+// hops and multiplies them like the blocks, see build_coarse_from).
+template <int NV, typename R>
 __global__ void __launch_bounds__(256) face_kernel(double2 *__restrict__ F, const C<R> *__restrict__ Q,
-                                                   const C<R> *__restrict__ U, const double2 *__restrict__ Yf,
-                                                   Geom g, FaceMap m, int chf) {
+                                                   const double2 *__restrict__ Yf, Geom g, FaceMap m, int chf) {
     extern __shared__ unsigned char sm_raw[];
     C<R> *sm = reinterpret_cast<C<R> *>(sm_raw);
     const int run = m.run;
@@ -183,21 +182,14 @@ __global__ void __launch_bounds__(256) face_kernel(double2 *__restrict__ F, cons
             int s;
             face_site(m, xc, mu, dir, f, site, s);
             const C<R> *ql = Q + (int64_t)l * m.nelem;
-            if (FINE) {
-                for (int e = 0; e < 12; ++e) a[e] = ql[(site * 12 + e) * m.Ls + s];
-                C<R> acc12[12];
-                fine_face_hop<R>(acc12, ql, U, g, m.Ls, site, s, mu, dir);
-                for (int e = 0; e < 12; ++e) h[e] = acc12[e];
-            } else {
-                for (int e = 0; e < run; ++e) a[e] = ql[site * run + e];
-                int64_t nb = shift_site(g, site, mu, dir);
-                const double2 *Yrow = Yf + (site * 9 + 1 + dd) * (int64_t)run * run;
-                const C<R> *qn = ql + nb * run;
-                for (int e = 0; e < run; ++e) {
-                    C<R> z = mk<R>(0, 0);
-                    for (int m2 = 0; m2 < run; ++m2) cfma(z, cvt<C<R>, double2>(Yrow[e * run + m2]), qn[m2]);
-                    h[e] = z;
-                }
+            for (int e = 0; e < run; ++e) a[e] = ql[site * run + e];
+            int64_t nb = shift_site(g, site, mu, dir);
+            const double2 *Yrow = Yf + (site * 9 + 1 + dd) * (int64_t)run * run;
+            const C<R> *qn = ql + nb * run;
+            for (int e = 0; e < run; ++e) {
+                C<R> z = mk<R>(0, 0);
+                for (int m2 = 0; m2 < run; ++m2) cfma(z, cvt<C<R>, double2>(Yrow[e * run + m2]), qn[m2]);
+                h[e] = z;
             }
         }
         __syncthreads();
@@ -219,6 +211,36 @@ __global__ void __launch_bounds__(256) face_kernel(double2 *__restrict__ F, cons
     for (int q = 0; q < PPT; ++q) {
         int p = threadIdx.x + q * 256;
         if (p < NP) F[(xc * 8 + dd) * NP + p] = acc[q];
+    }
+}
+
+// face element f = i*Ls + s of block xc for (mu, dir): its fine site
+__device__ __forceinline__ int64_t face_elem_site(const FaceMap &m, int64_t xc, int mu, int dir, int64_t f, int &s) {
+    int64_t site;
+    face_site(m, xc, mu, dir, f, site, s);
+    return site;
+}
+
+// Hf[dd - dd0][l][xc][(i*12 + e)*Ls + s] = the hop T_{1+dd}(q_l) at face element
+// (i, s) of block xc, dd = dd0 + blockIdx.y
+template <typename R>
+__global__ void __launch_bounds__(256) face_terms_kernel(C<R> *__restrict__ Hf, const C<R> *__restrict__ Q,
+                                                         const C<R> *__restrict__ U, Geom g, FaceMap m, int64_t nc,
+                                                         int64_t nfe, int dd0) {
+    const int64_t xc = blockIdx.x;
+    const int dd = dd0 + blockIdx.y, l = blockIdx.z;
+    const int mu = dd >> 1, dir = (dd & 1) ? -1 : +1;
+    const int nv = gridDim.z;
+    const int64_t nface = (int64_t)m.b[0] * m.b[1] * m.b[2] * m.b[3] / m.b[mu] * m.Ls;
+    const C<R> *ql = Q + (int64_t)l * m.nelem;
+    C<R> *out = Hf + (((int64_t)blockIdx.y * nv + l) * nc + xc) * nfe;
+    for (int64_t f = threadIdx.x; f < nface; f += blockDim.x) {
+        int s;
+        const int64_t site = face_elem_site(m, xc, mu, dir, f, s);
+        C<R> h[12];
+        fine_face_hop<R>(h, ql, U, g, m.Ls, site, s, mu, dir);
+        const int64_t i = f / m.Ls;
+        for (int e = 0; e < 12; ++e) out[(i * 12 + e) * m.Ls + s] = h[e];
     }
 }
 
@@ -340,19 +362,34 @@ template <typename R> void build_coarse_from(dwf_ctx *c, Level &L, Level &Lc, co
     m.Ls = L.lg.g.Ls;
     m.run = L.lg.ncomp;
     m.nelem = L.lg.nelem;
-    int chf = (int)std::max<int64_t>(1, (46 * 1024) / ((int64_t)2 * nv * m.run * sizeof(C<R>)));
-    size_t smem = (size_t)2 * nv * chf * m.run * sizeof(C<R>);
-    dim3 grid((unsigned)nc, 8);
-    bool fine = (L.index == 0);
-    const C<R> *Ul = std::is_same<R, double>::value ? (const C<R> *)c->U64.p : (const C<R> *)c->U32.p;
-#define FK(NV)                                                                                               \
-    if (fine) face_kernel<NV, true, R><<<grid, 256, smem, c->stream>>>(L.F.as<double2>(), Q, Ul, nullptr,     \
-                                                                      L.lg.g, m, chf);                       \
-    else face_kernel<NV, false, R><<<grid, 256, smem, c->stream>>>(L.F.as<double2>(), Q, nullptr,            \
-                                                                  L.Y64.as<double2>(), L.lg.g, m, chf)
-    NV_DISPATCH2(nv, FK);
+    if (L.index == 0) {
+        // The hops that leave a block, one direction mu at a time (both signs
+        // where they fit), stored in W, which the Gram matrix above was the
+        // last to read, and multiplied with the basis on the faces by the
+        // kernel of the block products: computing them inside the product
+        // kernel took 12.3 ms at Nvec 24, 12^3 x 16 x 16; this takes 2.5 ms
+        const C<R> *Ul = std::is_same<R, double>::value ? (const C<R> *)c->U64.p : (const C<R> *)c->U32.p;
+        for (int mu = 0; mu < 4; ++mu) {
+            const int64_t nfe = L.lg.nelem / nc / m.b[mu], hs = nc * nfe;
+            const int at_once = m.b[mu] > 1 ? 2 : 1;
+            for (int d0 = 0; d0 < 2; d0 += at_once) {
+                face_terms_kernel<R><<<dim3((unsigned)nc, (unsigned)at_once, (unsigned)nv), 256, 0, c->stream>>>(
+                    W, Q, Ul, L.lg.g, m, nc, nfe, 2 * mu + d0);
+                DWF_CHECK_LAUNCH();
+                for (int d = d0; d < d0 + at_once; ++d)
+                    face_gram<R>(c, L, L.F.as<double2>(), Q, W + (int64_t)(d - d0) * nv * hs, hs, mu, d == 0 ? +1 : -1);
+            }
+        }
+    } else {
+        int chf = (int)std::max<int64_t>(1, (46 * 1024) / ((int64_t)2 * nv * m.run * sizeof(C<R>)));
+        size_t smem = (size_t)2 * nv * chf * m.run * sizeof(C<R>);
+        dim3 grid((unsigned)nc, 8);
+#define FK(NV) \
+    face_kernel<NV, R><<<grid, 256, smem, c->stream>>>(L.F.as<double2>(), Q, L.Y64.as<double2>(), L.lg.g, m, chf)
+        NV_DISPATCH2(nv, FK);
 #undef FK
-    DWF_CHECK_LAUNCH();
+        DWF_CHECK_LAUNCH();
+    }
     size_t yb = sizeof(double2) * nc * 9 * np;
     if (Lc.Y64.bytes < yb) Lc.Y64.alloc(yb);
     unsigned blocks = (unsigned)std::min<int64_t>((nc * np + 255) / 256, (int64_t)c->sm_count * 16);
@@ -408,35 +445,6 @@ PairTable make_pairs() {
         }
     if (n != SQ_PAIRS) throw Error{DWF_ECUDA, "squared coarse stencil: pair table size"};
     return t;
-}
-
-// face element f = i*Ls + s of block xc for (mu, dir): its fine site
-__device__ __forceinline__ int64_t face_elem_site(const FaceMap &m, int64_t xc, int mu, int dir, int64_t f, int &s) {
-    int64_t site;
-    face_site(m, xc, mu, dir, f, site, s);
-    return site;
-}
-
-// Hf[dd][l][xc][(i*12 + e)*Ls + s] = T_{1+dd}(q_l) at face element (i, s) of block xc
-template <typename R>
-__global__ void __launch_bounds__(256) face_terms_kernel(C<R> *__restrict__ Hf, const C<R> *__restrict__ Q,
-                                                         const C<R> *__restrict__ U, Geom g, FaceMap m, int64_t nc,
-                                                         int64_t nfe) {
-    const int64_t xc = blockIdx.x;
-    const int dd = blockIdx.y, l = blockIdx.z;
-    const int mu = dd >> 1, dir = (dd & 1) ? -1 : +1;
-    const int nv = gridDim.z;
-    const int64_t nface = (int64_t)m.b[0] * m.b[1] * m.b[2] * m.b[3] / m.b[mu] * m.Ls;
-    const C<R> *ql = Q + (int64_t)l * m.nelem;
-    C<R> *out = Hf + (((int64_t)dd * nv + l) * nc + xc) * nfe;
-    for (int64_t f = threadIdx.x; f < nface; f += blockDim.x) {
-        int s;
-        const int64_t site = face_elem_site(m, xc, mu, dir, f, s);
-        C<R> h[12];
-        fine_face_hop<R>(h, ql, U, g, m.Ls, site, s, mu, dir);
-        const int64_t i = f / m.Ls;
-        for (int e = 0; e < 12; ++e) out[(i * 12 + e) * m.Ls + s] = h[e];
-    }
 }
 
 // W_l -= T_{1+dd}(q_l) on the face of every block (one dd per launch: no two
@@ -635,7 +643,7 @@ template <typename R> void build_squared_coarse(dwf_ctx *c, Level &L, Level &Lc,
     DevBuf Hf(sizeof(C<R>) * (size_t)(8 * nv * nc * nfe));
     const C<R> *Ul = std::is_same<R, double>::value ? (const C<R> *)c->U64.p : (const C<R> *)c->U32.p;
     face_terms_kernel<R><<<dim3((unsigned)nc, 8, (unsigned)nv), 256, 0, c->stream>>>(Hf.as<C<R>>(), Q, Ul, L.lg.g, m,
-                                                                                      nc, nfe);
+                                                                                      nc, nfe, 0);
     DWF_CHECK_LAUNCH();
     for (int dd = 0; dd < 8; ++dd) {
         if (m.L[dd >> 1] == 1) {

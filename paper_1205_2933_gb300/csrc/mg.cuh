@@ -38,7 +38,7 @@ struct Level {
     dwf_prec yprec = DWF_F64;
     // block reductions scratch: [Vc][nv][nv] complex FP64
     DevBuf G, F, Rinv;
-    DevBuf info;           // int per coarse site: Cholesky status
+    DevBuf info;           // int: set where a Cholesky pivot was lost
     // fused coarsest-level GCR: contiguous direction vectors, partial sums, counter
     DevBuf cgZ, cgW, cgPart, cgIters;
     // coarse levels: neighbour table int [V][npts - 1], entry 2 mu (+mu) and
@@ -87,7 +87,7 @@ void coarse_overlap_impl(dwf_ctx *c, int level, const double2 *f, int nf, double
 void mg_coarse_solve_impl(dwf_ctx *c, int level, void *x, const void *b);
 void mg_coarse_solve_static_impl(dwf_ctx *c, int level, void *x, const void *b);
 
-// ---- transfer.cu ----
+// ---- transfer.cu, block_setup.cu ----
 // c[Vc][nv] = R f  (R = P^+) ; f = P c (accumulate: f += P c)
 template <typename R> void restrict_(dwf_ctx *c, const Level &L, C<R> *cout, const C<R> *fin, const C<R> *Q);
 template <typename R> void prolong_(dwf_ctx *c, const Level &L, C<R> *fout, const C<R> *cin, const C<R> *Q, bool accumulate);
@@ -101,6 +101,11 @@ template <typename R>
 void prolong_batch(dwf_ctx *c, const Level &L, C<R> *fout, const C<R> *cin, const C<R> *Q, int nrhs, bool accumulate);
 // G[Vc][nv][nv] = block inner products <A_k, B_l> over each block (FP64 accumulate)
 template <typename R> void block_gram(dwf_ctx *c, const Level &L, double2 *G, const C<R> *A, const C<R> *B);
+// F[(Vc 8 + dd)][nv][nv] = <Q_k, H_l> over the face of each block in direction
+// mu (dir > 0: its last layer, dd = 2 mu; else the first, dd = 2 mu + 1), H
+// holding the faces alone, one block after another, vectors hstride apart
+template <typename R>
+void face_gram(dwf_ctx *c, const Level &L, double2 *F, const C<R> *Q, const C<R> *H, int64_t hstride, int mu, int dir);
 // In-place block orthonormalisation of the nv fields Q (CholQR2, FP64); returns false on breakdown
 template <typename R> bool block_orthonormalise(dwf_ctx *c, Level &L, C<R> *Q);
 // Q[2j] = (1 + Gamma)/2 v_j, Q[2j+1] = (1 - Gamma)/2 v_j  (Gamma = g5 R5 on the fine level,
@@ -178,6 +183,9 @@ void cg_combine_b(dwf_ctx *c, T *x, T *const *Z, int k, int base, int stride, in
 template <typename T>
 void cg_chunk_b(dwf_ctx *c, T *x, T *p, T *const *Z, int m, bool next, bool xinit, int base, int stride, int zb, int wb,
                 int k0, int rs, int64_t n, int nrhs);
+// out = x / |x| in FP64 for every right-hand side, |x|^2 in slot base + r*stride
+template <typename T>
+void normalised_b(dwf_ctx *c, double2 *out, const T *x, int base, int stride, int64_t n, int nrhs);
 template <typename T> void gcr_wr_b(dwf_ctx *c, T *w, T *res, const double *sc, const double2 *al, int64_t n, int nrhs);
 template <typename T> void combo_b(dwf_ctx *c, T *x, T *const *V, int k, const double2 *g, int64_t n, int nrhs);
 
