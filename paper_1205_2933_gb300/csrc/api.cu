@@ -109,6 +109,8 @@ dwf_status create_one(dwf_ctx **out, const int dims[4], int Ls, double M5, doubl
         c->g.Ls = Ls;
         c->g.V = (int64_t)dims[0] * dims[1] * dims[2] * dims[3];
         c->g.ap = antiperiodic_t ? 1 : 0;
+        if (dwf::dslash_pair_supported(Ls))
+            for (int w = 0; w < 2; ++w) c->brick[w] = dwf::pick_brick(c->g, (2 << w) * (32 / (Ls / 2)));
         c->M5 = M5;
         c->mf = mf;
         c->stream = (cudaStream_t)stream;

@@ -4,25 +4,12 @@
 
 #include <algorithm>
 
+#include "fastdiv.cuh"
 #include "mg.cuh"
 
 namespace dwf {
 
 namespace {
-
-// n / d for 0 <= n < 2^31 as a multiply-high, an addition and a shift
-struct FastDiv {
-    unsigned m;
-    int l, d;
-    __device__ __forceinline__ unsigned div(unsigned n) const { return (__umulhi(m, n) + n) >> l; }
-};
-
-FastDiv fast_div(int d) {
-    FastDiv f{0, 0, d};
-    while (((int64_t)1 << f.l) < d) ++f.l;
-    f.m = (unsigned)((((uint64_t)1 << 32) * (((uint64_t)1 << f.l) - (uint64_t)d)) / (uint64_t)d + 1);
-    return f;
-}
 
 // A box of finer sites (a block, or one face of it) taken in the order of its
 // sites, each with its contiguous run of elements.

@@ -216,12 +216,25 @@ void dslash(dwf_ctx *c, double2 *out, const double2 *in, bool dag, int nrhs) {
     c->applies64 += nrhs;
 }
 
-bool dslash_pair_supported(int Ls);
+// ---- the paired FP32 kernel (dslash_pair.cuh) ----
+template <int LS>
+void dslash_pair_ls(dwf_ctx *c, float2 *out, const float2 *in, bool dag, int nrhs, int minb, double *nslot, int nstride,
+                    const ZUpdate *zu);
+
 // zin with nslot: out = zin - a D^+ in (add: out = D in + a zin), a = zz[r * nstride] / ww[r * nstride]
 // per right-hand side r; zin without nslot: out = zin - D in
-void dslash_pair_f32(dwf_ctx *c, float2 *out, const float2 *in, bool dag, int nrhs, int minb, double *nslot,
-                     int nstride, const float2 *zin = nullptr, const double *zz = nullptr, const double *ww = nullptr,
-                     bool add = false);
+static void dslash_pair_f32(dwf_ctx *c, float2 *out, const float2 *in, bool dag, int nrhs, int minb, double *nslot,
+                            int nstride, const float2 *zin = nullptr, const double *zz = nullptr,
+                            const double *ww = nullptr, bool add = false) {
+    const ZUpdate zu{zin, zz, ww, nstride, add ? 1 : 0};
+    const ZUpdate *zp = zin ? &zu : nullptr;
+    switch (c->g.Ls) {
+#define LSC(L) case L: dslash_pair_ls<L>(c, out, in, dag, nrhs, minb, nslot, nstride, zp); break
+        LSC(4); LSC(6); LSC(8); LSC(10); LSC(12); LSC(16); LSC(20); LSC(24); LSC(32); LSC(48); LSC(64);
+#undef LSC
+        default: throw Error{DWF_EINVAL, "paired Dslash: fifth extent not instantiated"};
+    }
+}
 
 namespace {
 // two slices per thread with packed FP32x2 arithmetic where Ls allows;
@@ -240,7 +253,10 @@ int pair_minb() {
 
 void dslash(dwf_ctx *c, float2 *out, const float2 *in, bool dag, int nrhs) {
     ProfScope ps(c, K_DSLASH_F32, nrhs);
-    if (pair_minb() && dslash_pair_supported(c->g.Ls)) {
+    // the paired kernel's 16-byte accesses need 16-byte aligned fields (an even
+    // Ls keeps every row of an aligned field aligned)
+    const bool aligned = (((uintptr_t)out | (uintptr_t)in) & 15) == 0;
+    if (pair_minb() && dslash_pair_supported(c->g.Ls) && aligned) {
         dslash_pair_f32(c, out, in, dag, nrhs, pair_minb(), nullptr, 0);
         c->applies32 += nrhs;
         return;

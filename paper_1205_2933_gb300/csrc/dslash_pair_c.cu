@@ -1,0 +1,10 @@
+// The paired FP32 Dslash for Ls = 6, 10, 12 (see dslash_pair.cuh).
+#include "dslash_pair.cuh"
+
+namespace dwf {
+
+template void dslash_pair_ls<6>(dwf_ctx *, float2 *, const float2 *, bool, int, int, double *, int, const ZUpdate *);
+template void dslash_pair_ls<10>(dwf_ctx *, float2 *, const float2 *, bool, int, int, double *, int, const ZUpdate *);
+template void dslash_pair_ls<12>(dwf_ctx *, float2 *, const float2 *, bool, int, int, double *, int, const ZUpdate *);
+
+}  // namespace dwf

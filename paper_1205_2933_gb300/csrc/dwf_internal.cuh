@@ -6,11 +6,13 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <array>
 #include <string>
 #include <vector>
 
 #include "dwfmg.h"
+#include "fastdiv.cuh"
 
 namespace dwf {
 
@@ -139,6 +141,63 @@ __host__ __device__ __forceinline__ int64_t site_index(const Geom &g, const int 
     return (((int64_t)c[3] * g.L[2] + c[2]) * g.L[1] + c[1]) * g.L[0] + c[0];
 }
 
+// The sites of one CTA of the paired FP32 Dslash (dslash_pair.cuh).
+struct Brick {
+    int b[4];         // extents
+    FastDiv db[3];    // ... the division by the first three
+    FastDiv dn[3];    // division by the bricks per lattice row in x, y, z
+    int64_t count;    // bricks of the lattice (the last ones of a row may overhang)
+};
+
+// the brick of at most `sites` sites that needs the fewest CTAs; among these the
+// one with the longest x extent up to 4, then y, z
+inline Brick pick_brick(const Geom &g, int sites) {
+    int best[4] = {1, 1, 1, 1};
+    int64_t ctas = -1;
+    int b[4];
+    for (b[0] = std::min({sites, g.L[0], 4}); b[0] >= 1; --b[0])
+        for (b[1] = std::min(sites / b[0], g.L[1]); b[1] >= 1; --b[1])
+            for (b[2] = std::min(sites / (b[0] * b[1]), g.L[2]); b[2] >= 1; --b[2]) {
+                b[3] = std::min(sites / (b[0] * b[1] * b[2]), g.L[3]);
+                int64_t n = 1;
+                for (int i = 0; i < 4; ++i) n *= (g.L[i] + b[i] - 1) / b[i];
+                if (ctas < 0 || n < ctas) {
+                    ctas = n;
+                    for (int i = 0; i < 4; ++i) best[i] = b[i];
+                }
+            }
+    Brick k;
+    k.count = 1;
+    for (int i = 0; i < 4; ++i) {
+        const int nb = (g.L[i] + best[i] - 1) / best[i];
+        k.b[i] = best[i];
+        k.count *= nb;
+        if (i < 3) {
+            k.db[i] = fast_div(best[i]);
+            k.dn[i] = fast_div(nb);
+        }
+    }
+    return k;
+}
+
+// The normal-equations residual update of CGNR, z <- z - a D^+ w, with
+// a = zz / ww of each right-hand side read from the scalar slots.
+struct ZUpdate {
+    const float2 *zin;  // the second field (not the output buffer)
+    const double *zz;   // numerator of a for right-hand side r at zz[r * stride]
+    const double *ww;   // denominator of a at ww[r * stride]
+    int stride;
+    int add;            // 1: out = D in + a zin (EPI 4); 0: out = zin - a D^+ in (EPI 2)
+};
+
+// fifth extents of the paired FP32 Dslash, and its sites per warp there
+inline bool dslash_pair_supported(int Ls) {
+    switch (Ls) {
+        case 4: case 6: case 8: case 10: case 12: case 16: case 20: case 24: case 32: case 48: case 64: return true;
+        default: return false;
+    }
+}
+
 // Device scalar slots used by solver kernels (coefficients stay on the GPU).
 constexpr int NSCALAR = 8192;
 
@@ -178,6 +237,7 @@ struct dwf_ctx {
     int device = 0;
     int sm_count = 0;
     dwf_status sticky = DWF_OK;
+    dwf::Brick brick[2];  // of the paired Dslash with 64 and 128 threads per CTA
     // links: FP64 full 3x3 [V][4][3][3]; FP32 two rows [V][4][2][3]
     dwf::DevBuf U64, U32;
     // device scalars (double), pinned host mirror
