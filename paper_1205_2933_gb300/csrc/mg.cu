@@ -616,13 +616,15 @@ template <typename R> class BatchRunner {
     int nr;
     Runner<R> one;
     static constexpr int SB = 1024, SS = 160;  // per-RHS scalar slot blocks: SB + r*SS
-    DevBuf dcoef;                              // per-RHS coefficient arrays (device)
 
     BatchRunner(dwf_ctx *ctx, MGState &m, int nrhs) : c(ctx), mg(m), nr(nrhs), one(ctx, m) {
         DWF_REQUIRE(SB + nr * SS <= NSCALAR, DWF_EINVAL, "too many right-hand sides in one batch");
         mg.bscratch.ensure(nr);
-        dcoef.alloc(sizeof(double2) * (size_t)nr * (MAX_RESTART + 2));
-        dscale.alloc(sizeof(double) * (size_t)nr);
+        grow(mg.bcoef, sizeof(double2) * (size_t)nr * (MAX_RESTART + 2));
+        grow(mg.bscale, sizeof(double) * (size_t)nr);
+    }
+    static void grow(DevBuf &b, size_t bytes) {
+        if (b.bytes < bytes) b.alloc(bytes);
     }
 
     int64_t n(int l) const { return mg.lev[l].lg.nelem; }
@@ -921,12 +923,9 @@ template <typename R> class BatchRunner {
     // Coarsest-level solves of every right-hand side.  One fused solve fills
     // about a third of the SMs, so NS of them run at a time on side streams
     // (each with its own scratch), joined back to the context stream.
-    static constexpr int NS = 3;
+    static constexpr int NS = MGState::NSIDE;
     cudaStream_t side[NS] = {nullptr, nullptr, nullptr};
     cudaEvent_t ev_fork = nullptr, ev_join[NS] = {nullptr, nullptr, nullptr};
-    DevBuf cs_r[NS], cs_Z[NS], cs_W[NS], cs_part[NS];
-
-    DevBuf cb_r, cb_Z, cb_W, cb_part;  // scratch of the batched coarsest solver
 
     void coarse_solves(T *x2, const T *b2, int64_t Nc) {
         Level &Lc = mg.lev[1];
@@ -935,24 +934,27 @@ template <typename R> class BatchRunner {
             const char *e = getenv("DWF_COARSE_BATCH");
             return !(e && atoi(e) == 0);
         }();
+        if (nr == 1) {
+            // one right-hand side: the fused solver of one (no lockstep, no grid tuning)
+            one.coarse_solve(1, x2, b2);
+            return;
+        }
         if (batched && coarse_gcr_batch_ok(Lc, p.coarse_restart, std::min(nr, 16))) {
             // all right-hand sides through one cooperative launch (16 at a time)
             const int w = std::min(nr, 16);
             const size_t vb = sizeof(T) * (size_t)Nc * w;
-            if (cb_r.bytes < vb) {
-                cb_r.alloc(vb);
-                cb_Z.alloc(vb * p.coarse_restart);
-                cb_W.alloc(vb * p.coarse_restart);
-            }
-            if (!cb_part.p) cb_part.alloc(coarse_gcr_batch_part_bytes(c));
+            grow(mg.cb_r, vb);
+            grow(mg.cb_Z, vb * p.coarse_restart);
+            grow(mg.cb_W, vb * p.coarse_restart);
+            grow(mg.cb_part, coarse_gcr_batch_part_bytes(c));
             if (!Lc.cgIters.p) {
                 Lc.cgIters.alloc(sizeof(int));
                 DWF_CUDA(cudaMemsetAsync(Lc.cgIters.p, 0, sizeof(int), c->stream));
             }
             for (int r0 = 0; r0 < nr; r0 += w) {
                 const int nb = std::min(w, nr - r0);
-                coarse_gcr_fused_batch<R>(c, Lc, x2 + (size_t)r0 * Nc, b2 + (size_t)r0 * Nc, nb, cb_r.as<T>(),
-                                          cb_Z.as<T>(), cb_W.as<T>(), cb_part.as<double2>(), Lc.cgIters.as<int>(),
+                coarse_gcr_fused_batch<R>(c, Lc, x2 + (size_t)r0 * Nc, b2 + (size_t)r0 * Nc, nb, mg.cb_r.as<T>(),
+                                          mg.cb_Z.as<T>(), mg.cb_W.as<T>(), mg.cb_part.as<double2>(), Lc.cgIters.as<int>(),
                                           p.coarsest_tol, p.coarsest_maxiter, p.coarse_restart);
             }
             return;
@@ -965,10 +967,10 @@ template <typename R> class BatchRunner {
             for (int i = 0; i < NS; ++i) {
                 DWF_CUDA(cudaStreamCreateWithFlags(&side[i], cudaStreamNonBlocking));
                 DWF_CUDA(cudaEventCreateWithFlags(&ev_join[i], cudaEventDisableTiming));
-                cs_r[i].alloc(sizeof(T) * Nc);
-                cs_Z[i].alloc(sizeof(T) * Nc * p.coarse_restart);
-                cs_W[i].alloc(sizeof(T) * Nc * p.coarse_restart);
-                cs_part[i].alloc(coarse_gcr_part_bytes(c));
+                grow(mg.cs_r[i], sizeof(T) * Nc);
+                grow(mg.cs_Z[i], sizeof(T) * Nc * p.coarse_restart);
+                grow(mg.cs_W[i], sizeof(T) * Nc * p.coarse_restart);
+                grow(mg.cs_part[i], coarse_gcr_part_bytes(c));
             }
             DWF_CUDA(cudaEventCreateWithFlags(&ev_fork, cudaEventDisableTiming));
             if (!Lc.cgIters.p) {
@@ -982,8 +984,8 @@ template <typename R> class BatchRunner {
         for (int r = 0; r < nr; ++r) {
             const int i = r % NS;
             c->stream = side[i];
-            coarse_gcr_fused<R>(c, Lc, x2 + (size_t)r * Nc, b2 + (size_t)r * Nc, cs_r[i].as<T>(), cs_Z[i].as<T>(),
-                                cs_W[i].as<T>(), cs_part[i].as<double2>(), Lc.cgIters.as<int>(), p.coarsest_tol,
+            coarse_gcr_fused<R>(c, Lc, x2 + (size_t)r * Nc, b2 + (size_t)r * Nc, mg.cs_r[i].as<T>(),
+                                mg.cs_Z[i].as<T>(), mg.cs_W[i].as<T>(), mg.cs_part[i].as<double2>(), Lc.cgIters.as<int>(), p.coarsest_tol,
                                 p.coarsest_maxiter, p.coarse_restart);
         }
         c->stream = main;
@@ -1218,9 +1220,9 @@ template <typename R> class BatchRunner {
                 }
                 alpha[(size_t)r * restart + k] = al[r];
             }
-            DWF_CUDA(cudaMemcpyAsync(dcoef.p, al.data(), sizeof(double2) * nr, cudaMemcpyHostToDevice, c->stream));
-            DWF_CUDA(cudaMemcpyAsync(dscale.p, scr.data(), sizeof(double) * nr, cudaMemcpyHostToDevice, c->stream));
-            gcr_wr_b<T>(c, W[k], rr, dscale.as<double>(), dcoef.as<double2>(), N, nr);
+            DWF_CUDA(cudaMemcpyAsync(mg.bcoef.p, al.data(), sizeof(double2) * nr, cudaMemcpyHostToDevice, c->stream));
+            DWF_CUDA(cudaMemcpyAsync(mg.bscale.p, scr.data(), sizeof(double) * nr, cudaMemcpyHostToDevice, c->stream));
+            gcr_wr_b<T>(c, W[k], rr, mg.bscale.as<double>(), mg.bcoef.as<double2>(), N, nr);
             for (int r = 0; r < nr; ++r)
                 if (act[r] && rn[r] <= tol[r] * bn[r]) act[r] = 0;
             ++k;
@@ -1242,8 +1244,8 @@ template <typename R> class BatchRunner {
                     g[(size_t)r * k + i] = make_double2(s.x / d, s.y / d);
                 }
             }
-            DWF_CUDA(cudaMemcpyAsync(dcoef.p, g.data(), sizeof(double2) * g.size(), cudaMemcpyHostToDevice, c->stream));
-            combo_b<T>(c, x, Z.data(), k, dcoef.as<double2>(), N, nr);
+            DWF_CUDA(cudaMemcpyAsync(mg.bcoef.p, g.data(), sizeof(double2) * g.size(), cudaMemcpyHostToDevice, c->stream));
+            combo_b<T>(c, x, Z.data(), k, mg.bcoef.as<double2>(), N, nr);
         }
         return active_iters;
     }
@@ -1302,7 +1304,9 @@ template <typename R> class BatchRunner {
                 if (rn[r] > tol * bn[r]) idx.push_back(r);
             const int na = (int)idx.size();
             if (na == 0) break;
-            if (cycles * p.outer_restart >= p.outer_maxiter) {
+            // the iteration limit: exact for one right-hand side, checked per cycle for a batch
+            const int left = nfull == 1 ? p.outer_maxiter - (int)iters : p.outer_maxiter - cycles * p.outer_restart;
+            if (left <= 0) {
                 status = DWF_ENOCONV;
                 break;
             }
@@ -1316,7 +1320,7 @@ template <typename R> class BatchRunner {
             nr = na;
             long long gi = 0;
             try {
-                gi = gcr_b(eR, bR, tin, std::min(p.outer_restart, 32));
+                gi = gcr_b(eR, bR, tin, std::min({p.outer_restart, 32, nfull == 1 ? left : 32}));
             } catch (...) {
                 nr = nfull;
                 throw;
@@ -1353,7 +1357,6 @@ template <typename R> class BatchRunner {
         return v[i].as<double2>();
     }
 
-    DevBuf dscale;  // per-RHS real scale factors (device)
 };
 
 bool batch_on() {
@@ -1364,15 +1367,18 @@ bool batch_on() {
     return on;
 }
 
+// The batched path covers FP32 V-cycles on two levels with nu_1 = 0, one
+// right-hand side included (its smoother then needs 2 launches per step instead
+// of 6: a V-cycle at 8^3 x 16 x 16 in 1.07 ms instead of 1.50); an FP16 basis copy is used only
+// by the one-at-a-time V-cycle.  DWF_BATCH=0 in the environment turns it off.
 template <typename R> bool batch_eligible(const MGState &mg, int nrhs) {
-    return std::is_same<R, float>::value && nrhs > 1 && batch_on() && mg.nlevels == 2 && mg.p.nu_pre == 0 &&
-           mg.p.outer_restart <= 32 && mg.p.coarsen == 0;
+    return std::is_same<R, float>::value && (nrhs > 1 || !mg.lev[0].Q16.p) && batch_on() && mg.nlevels == 2 &&
+           mg.p.nu_pre == 0 && mg.p.outer_restart <= 32 && mg.p.coarsen == 0;
 }
 
 // Right-hand sides per batch: at most 32, and no more than the free device
 // memory holds (9 + 2 * restart fine fields in precision R and two FP64
 // fields per right-hand side, counting the batch workspaces already held).
-// 1 means: solve one at a time.
 // The widest batch (at most 32, at most nrhs) whose fine-level workspaces fit
 // in 90% of the free device memory.  A workspace already held is reused when
 // it is large enough and replaced when it is not (the old one is freed
@@ -1396,8 +1402,8 @@ template <typename R> int batch_width(const MGState &mg, int nrhs, bool solve) {
     size_t fr = 0, tot = 0;
     DWF_CUDA(cudaMemGetInfo(&fr, &tot));
     int nb = std::min(32, nrhs);
-    while (nb > 1 && growth(nb) > 0.9 * (double)fr) --nb;
-    return nb;
+    while (nb >= 1 && growth(nb) > 0.9 * (double)fr) --nb;
+    return nb;  // 0: not even one
 }
 
 template <typename R>
@@ -1422,19 +1428,22 @@ dwf_status setup_t(dwf_ctx *c, MGState &mg, int levels, const void *start, bool 
     return DWF_OK;
 }
 
-// The batched path covers FP32 V-cycles on two levels with nu_1 = 0;
-// DWF_BATCH=0 in the environment turns it off.
 template <typename R>
 dwf_status solve_t(dwf_ctx *c, MGState &mg, double2 *b, double2 *x, double tol, int nrhs, mg_stats &st) {
-    int width = batch_eligible<R>(mg, nrhs) ? batch_width<R>(mg, nrhs, true) : 1;
+    // the width of the batches (0: one at a time without the batched path)
+    auto fitting = [&] {
+        const int w = batch_width<R>(mg, nrhs, true);
+        return w > 1 || nrhs == 1 ? w : 0;
+    };
+    int width = batch_eligible<R>(mg, nrhs) ? fitting() : 0;
     if (batch_eligible<R>(mg, nrhs) && width < std::min(nrhs, 32) && !mg.wsb[0].empty()) {
         // memory-bound: the workspaces another width left (e.g. the setup's
         // relaxation of all start vectors) give way to the solve's own
         for (int l = 0; l < MAX_LEVELS; ++l) mg.wsb[l].clear();
         mg.wsb64.clear();
-        width = batch_width<R>(mg, nrhs, true);
+        width = fitting();
     }
-    if (width > 1) {
+    if (width > 0) {
         const int64_t N = mg.lev[0].lg.nelem;
         dwf_status worst = DWF_OK;
         long long c0 = 0;
@@ -1677,8 +1686,9 @@ template <typename R> void coarse_solve_t(dwf_ctx *c, MGState &mg, int level, vo
 }
 template <typename R> void vcycle_t(dwf_ctx *c, MGState &mg, double2 *x, const double2 *b, int nrhs) {
     const int64_t N = mg.lev[0].lg.nelem;
-    const int width = batch_eligible<R>(mg, nrhs) ? batch_width<R>(mg, nrhs, false) : 1;
-    if (width > 1) {
+    int width = batch_eligible<R>(mg, nrhs) ? batch_width<R>(mg, nrhs, false) : 0;
+    if (width == 1 && nrhs > 1) width = 0;
+    if (width > 0) {
         for (int r0 = 0; r0 < nrhs; r0 += width) {
             const int nb = std::min(width, nrhs - r0);
             BatchRunner<R> br(c, mg, nb);

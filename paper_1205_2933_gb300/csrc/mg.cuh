@@ -61,6 +61,11 @@ struct MGState {
     // batched solve: nrhs-wide workspaces and reduction scratch
     std::vector<DevBuf> wsb[MAX_LEVELS], wsb64;
     BatchScratch bscratch;
+    // the batched solve's coefficient arrays and the scratch of its coarsest
+    // solves; kept between calls (every user runs on the context's stream)
+    DevBuf bcoef, bscale, cb_r, cb_Z, cb_W, cb_part;
+    static constexpr int NSIDE = 3;
+    DevBuf cs_r[NSIDE], cs_Z[NSIDE], cs_W[NSIDE], cs_part[NSIDE];
     mg_stats stats;
 };
 
