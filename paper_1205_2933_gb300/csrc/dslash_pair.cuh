@@ -251,6 +251,7 @@ dslash_pair_kernel(float2 *__restrict__ out0, const float2 *__restrict__ in0, co
     const bool active = brick_site(bk, g, blockIdx.x, ls, x) && wl < SPW;
     if (!active) x[0] = x[1] = x[2] = x[3] = 0;  // idle lanes compute on site 0 and store nothing
     const int site = site_of(g, x);
+    pdl_dependents();  // the next kernel's prologue may run beside this grid's tail
     // the links of the CTA's sites: U_mu(x) and U_mu(x-mu), two stored rows, the
     // third rebuilt as conj(row0 x row1) (det U = 1), scaled by the hop
     // coefficient and duplicated into (re, re, im, im)
@@ -289,6 +290,7 @@ dslash_pair_kernel(float2 *__restrict__ out0, const float2 *__restrict__ in0, co
 #pragma unroll
         for (int k = 0; k < 12; ++k) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(zp + k * LS));
     };
+    pdl_wait();  // the links are constant; fields and scalar slots are not
     if (EPI >= 2 && active) request_z(r0);
     __syncthreads();
     for (int rhs = r0; rhs < r1; ++rhs) {
@@ -383,6 +385,8 @@ dslash_pair_kernel(float2 *__restrict__ out0, const float2 *__restrict__ in0, co
 __global__ void __launch_bounds__(1024) norm_finish_kernel(const double *__restrict__ npart, double *__restrict__ nslot,
                                                            int nstride, int nb) {
     __shared__ double red[32];
+    pdl_dependents();
+    pdl_wait();
     const double *pr = npart + (size_t)blockIdx.x * nb;
     double t = 0;
     for (int i = threadIdx.x; i < nb; i += blockDim.x) t += pr[i];
@@ -432,8 +436,8 @@ void dslash_pair_ls(dwf_ctx *c, float2 *out, const float2 *in, bool dag, int nrh
     }
     const ZUpdate z = zu ? *zu : ZUpdate{nullptr, nullptr, nullptr, 0, 0};
 #define PL(D, E)                                                                                                  \
-    dslash_pair_kernel<D, LS, E><<<grid, threads, smem, c->stream>>>(out, in, U, g, bk, diag, mf, field, npart, z, \
-                                                                     nrhs, rb)
+    launch_after(dslash_pair_kernel<D, LS, E>, grid, dim3(threads), smem, c->stream, out, in, U, g, bk, diag, mf, \
+                 field, npart, z, nrhs, rb)
     if (zu && !nslot) PL(false, 3);
     else if (zu && zu->add) PL(false, 4);
     else if (zu) PL(true, 2);
@@ -444,7 +448,7 @@ void dslash_pair_ls(dwf_ctx *c, float2 *out, const float2 *in, bool dag, int nrh
 #undef PL
     DWF_CHECK_LAUNCH();
     if (nslot) {
-        norm_finish_kernel<<<nrhs, 1024, 0, c->stream>>>(npart, nslot, nstride, (int)grid.x);
+        launch_after(norm_finish_kernel, dim3(nrhs), dim3(1024), 0, c->stream, npart, nslot, nstride, (int)grid.x);
         DWF_CHECK_LAUNCH();
     }
 }

@@ -92,6 +92,30 @@ void note_launches(unsigned long long n);  // kernels launched by a replayed gra
         if (!(cond)) throw ::dwf::Error{code, text};                                          \
     } while (0)
 
+// Programmatic dependent launch: a kernel launched by launch_after may start
+// once every CTA of the kernel before it in the stream has called
+// pdl_dependents (or ended), and runs up to its pdl_wait beside that kernel's
+// tail; pdl_wait returns when the kernel before has completed and its writes
+// are visible.  Every such kernel calls pdl_wait before it touches anything a
+// kernel writes, so completion stays in stream order.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... K, typename... A>
+void launch_after(void (*fn)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    DWF_CUDA(cudaLaunchKernelEx(&cfg, fn, static_cast<K>(args)...));
+}
+
 // Owned device buffer.
 struct DevBuf {
     void *p = nullptr;
