@@ -401,6 +401,21 @@ __global__ void cg_chunk_b_kernel(T *__restrict__ x, T *__restrict__ p, MArgs<T>
     }
 }
 
+// p = zt + c (p - z), c = s[izt] / s[iz] (0 where the denominator is not positive)
+template <typename T>
+__global__ void cg_redirect_kernel(T *__restrict__ p, const T *__restrict__ zt, const T *__restrict__ z,
+                                   const double *__restrict__ s, int izt, int iz, int64_t n) {
+    using R = typename RealB<T>::type;
+    const R cf = s[iz] > 0.0 ? (R)(s[izt] / s[iz]) : R(0);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const T pv = p[i], zv = z[i], tv = zt[i];
+        T o;
+        o.x = tv.x + cf * (pv.x - zv.x);
+        o.y = tv.y + cf * (pv.y - zv.y);
+        p[i] = o;
+    }
+}
+
 dim3 grid_b(dwf_ctx *c, int64_t n, int nrhs, int cap_per_sm) {
     int64_t b = (n + BT - 1) / BT;
     int64_t cap = std::max<int64_t>(1, (int64_t)c->sm_count * cap_per_sm / std::max(1, nrhs));
@@ -552,6 +567,12 @@ void cg_chunk_b(dwf_ctx *c, T *x, T *p, T *const *Z, int m, bool next, bool xini
     DWF_CHECK_LAUNCH();
 }
 
+template <typename T>
+void cg_redirect(dwf_ctx *c, T *p, const T *zt, const T *z, int izt, int iz, int64_t n) {
+    cg_redirect_kernel<T><<<grid_b(c, n, 1, 16), BT, 0, c->stream>>>(p, zt, z, c->scal.as<double>(), izt, iz, n);
+    DWF_CHECK_LAUNCH();
+}
+
 #define INSTB(T)                                                                                            \
     template void norm2_b<T>(dwf_ctx *, BatchScratch &, int, int, const T *, int64_t, int);                  \
     template void multidot_b<T>(dwf_ctx *, BatchScratch &, int, int, T *const *, int, const T *, int64_t, int); \
@@ -565,6 +586,7 @@ void cg_chunk_b(dwf_ctx *c, T *x, T *p, T *const *Z, int m, bool next, bool xini
     template void cg_chunk_b<T>(dwf_ctx *, T *, T *, T *const *, int, bool, bool, int, int, int, int, int, int,   \
                                 int64_t, int);                                                                 \
     template void normalised_b<T>(dwf_ctx *, double2 *, const T *, int, int, int64_t, int);                   \
+    template void cg_redirect<T>(dwf_ctx *, T *, const T *, const T *, int, int, int64_t);                   \
     template void gcr_wr_b<T>(dwf_ctx *, T *, T *, const double *, const double2 *, int64_t, int);            \
     template void combo_b<T>(dwf_ctx *, T *, T *const *, int, const double2 *, int64_t, int);
 INSTB(float2)

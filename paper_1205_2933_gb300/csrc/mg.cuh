@@ -191,6 +191,9 @@ void cg_chunk_b(dwf_ctx *c, T *x, T *p, T *const *Z, int m, bool next, bool xini
 // out = x / |x| in FP64 for every right-hand side, |x|^2 in slot base + r*stride
 template <typename T>
 void normalised_b(dwf_ctx *c, double2 *out, const T *x, int base, int stride, int64_t n, int nrhs);
+// a CG direction moved to a replaced residual: p = zt + c (p - z), c = |zt|^2 / |z|^2
+// from the slots izt, iz (with p = z + b p_old: zt + (|zt|^2 / |z_old|^2) p_old)
+template <typename T> void cg_redirect(dwf_ctx *c, T *p, const T *zt, const T *z, int izt, int iz, int64_t n);
 template <typename T> void gcr_wr_b(dwf_ctx *c, T *w, T *res, const double *sc, const double2 *al, int64_t n, int nrhs);
 template <typename T> void combo_b(dwf_ctx *c, T *x, T *const *V, int k, const double2 *g, int64_t n, int nrhs);
 
