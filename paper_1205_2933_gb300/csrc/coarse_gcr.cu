@@ -24,27 +24,27 @@ size_t coarse_gcr_part_bytes(dwf_ctx *c) { return sizeof(double2) * 3 * (MAXR + 
 
 template <typename R>
 static void launch_any(dwf_ctx *c, const Level &L, C<R> *x, const C<R> *b, C<R> *r, C<R> *Z, C<R> *W, double2 *part,
-                       int *iters, double tol, int maxiter, int restart) {
-    if (L.npts == 33) return coarse_gcr_launch_squared<R>(c, L, x, b, r, Z, W, part, iters, tol, maxiter, restart);
+                       int *iters, double tol, int maxiter, int restart, int max_ctas) {
+    if (L.npts == 33) return coarse_gcr_launch_squared<R>(c, L, x, b, r, Z, W, part, iters, tol, maxiter, restart, max_ctas);
     switch (L.yprec) {
-        case DWF_F64: launch_t<R, double2, 9>(c, L, L.Y64.as<double2>(), x, b, r, Z, W, part, iters, tol, maxiter, restart); break;
-        case DWF_F32: launch_t<R, float2, 9>(c, L, L.Y32.as<float2>(), x, b, r, Z, W, part, iters, tol, maxiter, restart); break;
-        case DWF_BF16: launch_t<R, __nv_bfloat162, 9>(c, L, L.Y16.as<__nv_bfloat162>(), x, b, r, Z, W, part, iters, tol, maxiter, restart); break;
-        case DWF_F16: launch_t<R, __half2, 9>(c, L, L.Y16.as<__half2>(), x, b, r, Z, W, part, iters, tol, maxiter, restart); break;
+        case DWF_F64: launch_t<R, double2, 9>(c, L, L.Y64.as<double2>(), x, b, r, Z, W, part, iters, tol, maxiter, restart, max_ctas); break;
+        case DWF_F32: launch_t<R, float2, 9>(c, L, L.Y32.as<float2>(), x, b, r, Z, W, part, iters, tol, maxiter, restart, max_ctas); break;
+        case DWF_BF16: launch_t<R, __nv_bfloat162, 9>(c, L, L.Y16.as<__nv_bfloat162>(), x, b, r, Z, W, part, iters, tol, maxiter, restart, max_ctas); break;
+        case DWF_F16: launch_t<R, __half2, 9>(c, L, L.Y16.as<__half2>(), x, b, r, Z, W, part, iters, tol, maxiter, restart, max_ctas); break;
     }
 }
 
 template <typename R>
 void coarse_gcr_fused(dwf_ctx *c, const Level &L, C<R> *x, const C<R> *b, C<R> *r, C<R> *Z, C<R> *W, double2 *part,
-                      int *iters, double tol, int maxiter, int restart) {
+                      int *iters, double tol, int maxiter, int restart, int max_ctas) {
     ProfScope ps(c, K_COARSE);
-    launch_any<R>(c, L, x, b, r, Z, W, part, iters, tol, maxiter, restart);
+    launch_any<R>(c, L, x, b, r, Z, W, part, iters, tol, maxiter, restart, max_ctas);
 }
 
 template void coarse_gcr_fused<double>(dwf_ctx *, const Level &, double2 *, const double2 *, double2 *, double2 *,
-                                       double2 *, double2 *, int *, double, int, int);
+                                       double2 *, double2 *, int *, double, int, int, int);
 template void coarse_gcr_fused<float>(dwf_ctx *, const Level &, float2 *, const float2 *, float2 *, float2 *, float2 *,
-                                      double2 *, int *, double, int, int);
+                                      double2 *, int *, double, int, int, int);
 
 }  // namespace dwf
 
@@ -110,7 +110,7 @@ static void static_solve_t(dwf_ctx *c, const Level &L, C<R> *x, const C<R> *b, d
     C<R> *W = Z + (size_t)restart * N;
     zero_int_kernel<<<1, 1, 0, c->stream>>>(iters);  // the counter must start at zero
     DWF_CHECK_LAUNCH();
-    launch_any<R>(c, L, x, b, r, Z, W, partials, iters, tol, maxiter, restart);
+    launch_any<R>(c, L, x, b, r, Z, W, partials, iters, tol, maxiter, restart, c->sm_count);
 }
 
 void mg_coarse_solve_static_impl(dwf_ctx *c, int level, void *x, const void *b) {

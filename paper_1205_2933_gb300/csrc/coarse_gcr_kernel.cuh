@@ -116,6 +116,8 @@ __device__ void gather_totals(const double2 *part, int k, int nb, double2 *tot) 
     __syncthreads();
 }
 
+// The solver with its vectors in global memory: for directions that do not fit
+// the SMs' shared memory (coarse_gcr_smem_kernel below takes the others).
 template <typename R, typename LT, int NV, int NPTS>
 __global__ void __launch_bounds__(CT) coarse_gcr_kernel(Args<R, LT> a) {
     cg::grid_group grid = cg::this_grid();
@@ -270,11 +272,311 @@ __global__ void __launch_bounds__(CT) coarse_gcr_kernel(Args<R, LT> a) {
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(a.iters, it);
 }
 
+// ---- the solver with its vectors in shared memory ---------------------------
+//
+// Sums that cross threads and CTAs: FP64 for FP64 fields; for FP32 fields the
+// unevaluated sum of two FP32 numbers (about 48 bits), because an FP64 addition
+// takes this chip's SM as long as 64 FP32 ones and every CTA adds up all
+// partials of a reduction.
+struct FF {
+    float hi, lo;
+};
+__device__ __forceinline__ void acc_init(FF &a) { a.hi = a.lo = 0.f; }
+__device__ __forceinline__ void acc_init(double &a) { a = 0.0; }
+__device__ __forceinline__ void acc_add(FF &a, FF b) {  // two-sum of the high parts
+    const float t = a.hi + b.hi, q = t - a.hi;
+    const float e = (a.hi - (t - q)) + (b.hi - q) + (a.lo + b.lo);
+    a.hi = t + e;
+    a.lo = e - (a.hi - t);
+}
+__device__ __forceinline__ void acc_add(double &a, double b) { a += b; }
+__device__ __forceinline__ void acc_fma(FF &a, float x, float y) {  // a += x y, the product exact
+    const float p = __fmul_rn(x, y);  // not contracted with the addition that follows
+    acc_add(a, FF{p, fmaf(x, y, -p)});
+}
+__device__ __forceinline__ void acc_fma(double &a, double x, double y) { a += x * y; }
+__device__ __forceinline__ FF acc_xor(FF a, int o) {
+    return FF{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+}
+__device__ __forceinline__ double acc_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ double acc_value(FF a) { return (double)a.hi + (double)a.lo; }
+__device__ __forceinline__ double acc_value(double a) { return a; }
+template <typename R> struct AccT;
+template <> struct AccT<float> { using type = FF; };
+template <> struct AccT<double> { using type = double; };
+template <typename A> struct alignas(16) AccC {  // a complex partial sum, one 16-byte access
+    A re, im;
+};
+
+// sites per CTA and shared-memory layout of the solver for V sites on at most `ctas` CTAs
+template <typename R, typename LT, int NV, int NPTS> struct SmemPlan {
+    static constexpr int LROW0 = NV * (int)sizeof(LT);                       // a link row
+    // an odd number of 16-byte units, so that the rows of 8 lanes lie in 8 bank groups
+    static constexpr int LROW = LROW0 % 32 == 0 ? LROW0 + 16 : LROW0;
+    int64_t spc;
+    size_t vec, stage, links, total;
+    bool cached;  // the links fit as well
+    SmemPlan(int64_t V, int restart, int64_t ctas, size_t limit) {
+        spc = (V + ctas - 1) / ctas;
+        vec = ((size_t)spc * NV * sizeof(C<R>) + 15) / 16 * 16;
+        stage = (size_t)spc * NPTS * NV * sizeof(C<R>);
+        stage = (stage + 15) / 16 * 16;
+        links = (size_t)spc * NPTS * NV * LROW;
+        const size_t base = vec * (2 * (size_t)restart + 2) + 2 * stage;
+        cached = base + links <= limit;
+        total = base + (cached ? links : 0);
+    }
+};
+
+template <typename R, typename LT, int NV> __device__ __forceinline__ C<R> row_times(const unsigned char *row, const C<R> *x) {
+    // NV links of one row in accesses of 16 bytes (8 where the row is no multiple)
+    constexpr int B = NV * sizeof(LT) % 16 == 0 ? 16 : 8;
+    constexpr int E = B / (int)sizeof(LT) > 0 ? B / (int)sizeof(LT) : 1;
+    struct alignas(B) Chunk {
+        LT e[E];
+    };
+    C<R> acc = mk<R>(0, 0);
+    constexpr int NCH = NV / E;
+    Chunk ch[NCH < 8 ? NCH : 8];
+#pragma unroll
+    for (int c0 = 0; c0 < NCH; c0 += 8) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (c0 + i < NCH) ch[i] = *reinterpret_cast<const Chunk *>(row + (size_t)(c0 + i) * sizeof(Chunk));
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (c0 + i < NCH)
+#pragma unroll
+                for (int j = 0; j < E; ++j)
+                    cfma(acc, LRead<LT>::template get<R>(ch[i].e, j), x[(c0 + i) * E + j]);
+    }
+    return acc;
+}
+
+// The same GCR, with what a CTA owns of every vector (the directions Z and W,
+// x, r) and, where they fit, its sites' links in shared memory: only the
+// vector the stencil acts on crosses CTAs, through a.r, and each iteration
+// leaves the chip's SMs twice: one grid barrier to publish that vector, one
+// for the reduction.  The products <W_i, w>, |w|^2 and <w, r> are reduced
+// together: with W orthonormal |w|^2 loses sum |<W_i, w>|^2 in the projection
+// and <w, r> does not change (r is orthogonal to the W_i).  Where the
+// projection took 3/4 or more of |w|^2, where that difference would lose
+// digits, a second one follows with a reduction of its own.  The stencil: one
+// thread per (direction, row) of a site, the neighbours' values staged.
+// Bound by the latency of the two barriers and of one L2 round trip after
+// each: 512 sites x 24 in BF16 44 us where the vectors in global memory, four
+// barriers per iteration and FP64 sums took 118; 256 sites x 16 in FP64 76 us
+// against 673.
+template <typename R, typename LT, int NV, int NPTS>
+__global__ void __launch_bounds__(CT) coarse_gcr_smem_kernel(Args<R, LT> a, int spc, int cached) {
+    using A = typename AccT<R>::type;
+    using P = SmemPlan<R, LT, NV, NPTS>;
+    cg::grid_group grid = cg::this_grid();
+    extern __shared__ __align__(16) unsigned char sm[];
+    __shared__ double2 tot[MAXR + 2];
+    const int nb = gridDim.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int s0 = blockIdx.x * spc, ns = max(0, min(spc, (int)a.g.V - s0)), own = ns * NV;
+    const int64_t e0 = (int64_t)s0 * NV;
+    const size_t vec = ((size_t)spc * NV * sizeof(C<R>) + 15) / 16 * 16;
+    const size_t stage = ((size_t)spc * NPTS * NV * sizeof(C<R>) + 15) / 16 * 16;
+    auto W = [&](int i) { return reinterpret_cast<C<R> *>(sm + vec * i); };
+    auto Z = [&](int i) { return reinterpret_cast<C<R> *>(sm + vec * (a.restart + i)); };
+    C<R> *x = reinterpret_cast<C<R> *>(sm + vec * 2 * a.restart), *r = reinterpret_cast<C<R> *>(sm + vec * (2 * a.restart + 1));
+    C<R> *sin = reinterpret_cast<C<R> *>(sm + vec * (2 * a.restart + 2));
+    C<R> *sp = reinterpret_cast<C<R> *>(sm + vec * (2 * a.restart + 2) + stage);
+    unsigned char *sl = sm + vec * (2 * a.restart + 2) + 2 * stage;
+    AccC<A> *part = reinterpret_cast<AccC<A> *>(a.part);
+    C<R> *pub = a.r;  // the published vector
+
+    if (cached) {
+        constexpr int WR = P::LROW0 / 4;  // 4-byte words of a link row
+        const unsigned *src = reinterpret_cast<const unsigned *>(a.Y + (int64_t)s0 * NPTS * NV * NV);
+        for (int i = tid; i < ns * NPTS * NV * WR; i += CT)
+            *reinterpret_cast<unsigned *>(sl + (size_t)(i / WR) * P::LROW + (i % WR) * 4) = src[i];
+    }
+    // dst = A pub on the CTA's sites (pub published and a grid barrier passed)
+    auto apply = [&](C<R> *dst) {
+        for (int i = tid; i < ns * NPTS * NV; i += CT) {
+            const int l = i % NV, sd = i / NV, d = sd % NPTS, site = s0 + sd / NPTS;
+            const int o = d > 0 ? a.nbr[(int64_t)site * (NPTS - 1) + d - 1] : site;
+            sin[i] = __ldcg(pub + (int64_t)o * NV + l);
+        }
+        __syncthreads();
+        for (int i = tid; i < ns * NPTS * NV; i += CT) {
+            const unsigned char *row = cached ? sl + (size_t)i * P::LROW
+                                              : reinterpret_cast<const unsigned char *>(a.Y + ((int64_t)s0 * NPTS * NV + i) * NV);
+            sp[i] = row_times<R, LT, NV>(row, sin + i / NV * NV);
+        }
+        __syncthreads();
+        for (int e = tid; e < own; e += CT) {
+            const int site = e / NV, k = e - site * NV;
+            C<R> v = sp[site * NPTS * NV + k];
+#pragma unroll
+            for (int d = 1; d < NPTS; ++d) v = v + sp[(site * NPTS + d) * NV + k];
+            dst[e] = v;
+        }
+        __syncthreads();
+    };
+    // tot[i] = the sum over all CTAs of <u_i, v_i>, i < n, u_i and v_i given by
+    // the index; the partials in region `reg`, which no CTA reads any more
+    auto reduce = [&](int n, int reg, auto u, auto v) {
+        AccC<A> *pr = part + (size_t)reg * (MAXR + 2) * nb;
+        for (int i = warp; i < n; i += CT / 32) {
+            const C<R> *ui = u(i), *vi = v(i);
+            AccC<A> s;
+            acc_init(s.re);
+            acc_init(s.im);
+            for (int e = lane; e < own; e += 32) {
+                const C<R> p = ui[e], q = vi[e];
+                acc_fma(s.re, p.x, q.x);
+                acc_fma(s.re, p.y, q.y);
+                acc_fma(s.im, p.x, q.y);
+                acc_fma(s.im, -p.y, q.x);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                acc_add(s.re, acc_xor(s.re, o));
+                acc_add(s.im, acc_xor(s.im, o));
+            }
+            if (lane == 0) pr[(size_t)i * nb + blockIdx.x] = s;
+        }
+        __threadfence();
+        grid.sync();
+        for (int i = warp; i < n; i += CT / 32) {
+            AccC<A> s;
+            acc_init(s.re);
+            acc_init(s.im);
+            for (int k = lane; k < nb; k += 32) {
+                const float4 w = __ldcg(reinterpret_cast<const float4 *>(pr + (size_t)i * nb + k));
+                const AccC<A> t = *reinterpret_cast<const AccC<A> *>(&w);
+                acc_add(s.re, t.re);
+                acc_add(s.im, t.im);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                acc_add(s.re, acc_xor(s.re, o));
+                acc_add(s.im, acc_xor(s.im, o));
+            }
+            if (lane == 0) tot[i] = make_double2(acc_value(s.re), acc_value(s.im));
+        }
+        __syncthreads();
+    };
+
+    for (int e = tid; e < own; e += CT) {
+        x[e] = mk<R>(0, 0);
+        const C<R> v = a.b[e0 + e];
+        r[e] = v;
+        pub[e0 + e] = v;
+    }
+    __syncthreads();
+    reduce(1, 0, [&](int) { return r; }, [&](int) { return r; });
+    const double bn2 = tot[0].x;
+    double rn2 = bn2;
+    int it = 0, k = 0;
+    if (bn2 > 0.0) {
+        const double stop = a.tol * a.tol * bn2;
+        while (it < a.maxiter && rn2 > stop) {
+            C<R> *w = W(k), *z = Z(k);
+            for (int e = tid; e < own; e += CT) z[e] = r[e];
+            __threadfence();
+            grid.sync();  // pub = r everywhere
+            apply(w);
+            // values 0 .. k-1: <W_i, w>; k: |w|^2; k + 1: <w, r>
+            auto U = [&](int i) { return i < k ? W(i) : w; };
+            auto V = [&](int i) { return i <= k ? w : r; };
+            double ww = 0.0, wrx = 0.0, wry = 0.0;
+            for (int pass = 0; pass < 2; ++pass) {
+                reduce(k + 2, pass, U, V);
+                ww = tot[k].x;
+                wrx = tot[k + 1].x;
+                wry = tot[k + 1].y;
+                if (k == 0) break;
+                double removed = 0.0;
+                for (int i = 0; i < k; ++i) removed += tot[i].x * tot[i].x + tot[i].y * tot[i].y;
+                for (int e = tid; e < own; e += CT) {
+                    C<R> wv = w[e], zv = z[e];
+                    for (int i = 0; i < k; ++i) {
+                        const C<R> m = mk<R>(-(R)tot[i].x, -(R)tot[i].y);
+                        cfma(wv, m, W(i)[e]);
+                        cfma(zv, m, Z(i)[e]);
+                    }
+                    w[e] = wv;
+                    z[e] = zv;
+                }
+                __syncthreads();  // tot is rewritten by the next reduction
+                const bool again = pass == 0 && removed >= 0.75 * ww;
+                ww -= removed;
+                if (!again) break;
+            }
+            if (!(ww > 0.0)) break;  // breakdown: same decision in every CTA
+            const double inv = 1.0 / sqrt(ww), ar = wrx * inv, ai = wry * inv;
+            const R sc = (R)inv;
+            const C<R> al = mk<R>((R)ar, (R)ai), mal = mk<R>(-(R)ar, -(R)ai);
+            for (int e = tid; e < own; e += CT) {
+                const C<R> zv = sc * z[e], wv = sc * w[e];
+                C<R> xv = x[e], rv = r[e];
+                cfma(xv, al, zv);
+                cfma(rv, mal, wv);
+                z[e] = zv;
+                w[e] = wv;
+                x[e] = xv;
+                r[e] = rv;
+                pub[e0 + e] = rv;  // every CTA is past its reading of pub (the reduction's barrier)
+            }
+            rn2 -= ar * ar + ai * ai;
+            ++it;
+            ++k;
+            __syncthreads();
+            if (k == a.restart || rn2 <= stop) {
+                // true residual r = b - A x
+                for (int e = tid; e < own; e += CT) pub[e0 + e] = x[e];
+                __threadfence();
+                grid.sync();
+                apply(r);
+                for (int e = tid; e < own; e += CT) {
+                    const C<R> v = a.b[e0 + e];
+                    r[e] = v - r[e];
+                }
+                __syncthreads();
+                reduce(1, 0, [&](int) { return r; }, [&](int) { return r; });
+                for (int e = tid; e < own; e += CT) pub[e0 + e] = r[e];
+                rn2 = tot[0].x;
+                k = 0;
+                __syncthreads();
+            }
+        }
+    }
+    for (int e = tid; e < own; e += CT) a.x[e0 + e] = x[e];
+    if (blockIdx.x == 0 && tid == 0) atomicAdd(a.iters, it);
+}
+
+// Whole sites per CTA, one CTA per SM: the vectors' slices in shared memory
+// where 2 restart + 2 of them and two stages of the stencil's inputs fit, the
+// links with them where those fit too.
+template <typename R, typename LT, int NV, int NPTS> void launch_nv(dwf_ctx *c, Args<R, LT> &a, int max_ctas) {
+    const SmemPlan<R, LT, NV, NPTS> plan(a.g.V, a.restart, max_ctas, (size_t)c->smem_optin - 4096);
+    if (plan.total <= (size_t)c->smem_optin - 4096) {
+        void *fn = (void *)coarse_gcr_smem_kernel<R, LT, NV, NPTS>;
+        DWF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.total));
+        int spc = (int)plan.spc, cached = plan.cached ? 1 : 0;
+        void *kargs[] = {&a, &spc, &cached};
+        DWF_CUDA(coop_launch(c, fn, dim3((unsigned)((a.g.V + spc - 1) / spc)), dim3(CT), kargs, plan.total));
+        return;
+    }
+    void *kargs[] = {&a};
+    const int64_t nblk = std::max<int64_t>(1, std::min<int64_t>((a.g.V * NV + CT - 1) / CT, c->sm_count));
+    void *fn = (void *)coarse_gcr_kernel<R, LT, NV, NPTS>;
+    int per_sm = 0;
+    DWF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, CT, 0));
+    DWF_REQUIRE(per_sm >= 1, DWF_ECUDA, "fused coarse solver cannot be co-resident");
+    DWF_CUDA(coop_launch(c, fn, dim3((unsigned)nblk), dim3(CT), kargs, 0));
+}
+
 // Launch the solver for a stencil of NPTS points (9: R D P; 33: the squared
-// operator's P^+ D^+ D P).
+// operator's P^+ D^+ D P) on at most max_ctas CTAs.
 template <typename R, typename LT, int NPTS>
 void launch_t(dwf_ctx *c, const Level &L, const LT *Y, C<R> *x, const C<R> *b, C<R> *r, C<R> *Z, C<R> *W,
-                     double2 *part, int *iters, double tol, int maxiter, int restart) {
+                     double2 *part, int *iters, double tol, int maxiter, int restart, int max_ctas) {
     Args<R, LT> a;
     a.Y = Y;
     a.nbr = L.nbr.as<int>();
@@ -289,29 +591,17 @@ void launch_t(dwf_ctx *c, const Level &L, const LT *Y, C<R> *x, const C<R> *b, C
     a.maxiter = maxiter;
     a.restart = restart;
     a.iters = iters;
-    void *kargs[] = {&a};
-    const int n = L.lg.ncomp;
-    const int64_t N = L.lg.g.V * n;
-    int64_t nblk = (N + CT - 1) / CT;
-    if (nblk > c->sm_count) nblk = c->sm_count;
-    if (nblk < 1) nblk = 1;
-    dim3 grid((unsigned)nblk), block(CT);
-    void *fn = nullptr;
-    switch (n) {
-        case 2: fn = (void *)coarse_gcr_kernel<R, LT, 2, NPTS>; break;
-        case 4: fn = (void *)coarse_gcr_kernel<R, LT, 4, NPTS>; break;
-        case 6: fn = (void *)coarse_gcr_kernel<R, LT, 6, NPTS>; break;
-        case 8: fn = (void *)coarse_gcr_kernel<R, LT, 8, NPTS>; break;
-        case 12: fn = (void *)coarse_gcr_kernel<R, LT, 12, NPTS>; break;
-        case 16: fn = (void *)coarse_gcr_kernel<R, LT, 16, NPTS>; break;
-        case 24: fn = (void *)coarse_gcr_kernel<R, LT, 24, NPTS>; break;
-        case 32: fn = (void *)coarse_gcr_kernel<R, LT, 32, NPTS>; break;
+    switch (L.lg.ncomp) {
+        case 2: launch_nv<R, LT, 2, NPTS>(c, a, max_ctas); break;
+        case 4: launch_nv<R, LT, 4, NPTS>(c, a, max_ctas); break;
+        case 6: launch_nv<R, LT, 6, NPTS>(c, a, max_ctas); break;
+        case 8: launch_nv<R, LT, 8, NPTS>(c, a, max_ctas); break;
+        case 12: launch_nv<R, LT, 12, NPTS>(c, a, max_ctas); break;
+        case 16: launch_nv<R, LT, 16, NPTS>(c, a, max_ctas); break;
+        case 24: launch_nv<R, LT, 24, NPTS>(c, a, max_ctas); break;
+        case 32: launch_nv<R, LT, 32, NPTS>(c, a, max_ctas); break;
         default: throw Error{DWF_EINVAL, "unsupported Nvec"};
     }
-    int per_sm = 0;
-    DWF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, CT, 0));
-    DWF_REQUIRE(per_sm >= 1, DWF_ECUDA, "fused coarse solver cannot be co-resident");
-    DWF_CUDA(coop_launch(c, fn, grid, block, kargs, 0));
     DWF_CHECK_LAUNCH();
 }
 

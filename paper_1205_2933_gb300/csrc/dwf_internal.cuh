@@ -260,6 +260,7 @@ struct dwf_ctx {
     cudaStream_t stream = nullptr;
     int device = 0;
     int sm_count = 0;
+    int smem_optin = 0;  // shared memory a CTA may opt in to
     dwf_status sticky = DWF_OK;
     dwf::Brick brick[2];  // of the paired Dslash with 64 and 128 threads per CTA
     // links: FP64 full 3x3 [V][4][3][3]; FP32 two rows [V][4][2][3]

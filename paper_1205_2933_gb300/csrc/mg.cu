@@ -324,7 +324,7 @@ template <typename R> class Runner {
                 DWF_CUDA(cudaMemsetAsync(L.cgIters.p, 0, sizeof(int), c->stream));
             }
             coarse_gcr_fused<R>(c, L, x, b, ws(l, 10), L.cgZ.as<T>(), L.cgW.as<T>(), L.cgPart.as<double2>(),
-                                L.cgIters.as<int>(), p.coarsest_tol, p.coarsest_maxiter, p.coarse_restart);
+                                L.cgIters.as<int>(), p.coarsest_tol, p.coarsest_maxiter, p.coarse_restart, c->sm_count);
             return;
         }
         if (!coarsest && p.cycle == 1) {
@@ -986,7 +986,7 @@ template <typename R> class BatchRunner {
             c->stream = side[i];
             coarse_gcr_fused<R>(c, Lc, x2 + (size_t)r * Nc, b2 + (size_t)r * Nc, mg.cs_r[i].as<T>(),
                                 mg.cs_Z[i].as<T>(), mg.cs_W[i].as<T>(), mg.cs_part[i].as<double2>(), Lc.cgIters.as<int>(), p.coarsest_tol,
-                                p.coarsest_maxiter, p.coarse_restart);
+                                p.coarsest_maxiter, p.coarse_restart, c->sm_count / NS);
         }
         c->stream = main;
         for (int i = 0; i < NS; ++i) {

@@ -137,7 +137,7 @@ bool coarse_gcr_fused_ok(const Level &L, int restart);
 // ---- coarse_gcr_sq.cu ---- the same kernel on the 33-point stencil
 template <typename R>
 void coarse_gcr_launch_squared(dwf_ctx *c, const Level &L, C<R> *x, const C<R> *b, C<R> *r, C<R> *Z, C<R> *W,
-                               double2 *part, int *iters, double tol, int maxiter, int restart);
+                               double2 *part, int *iters, double tol, int maxiter, int restart, int max_ctas);
 // ---- coarse_gcr_batch.cu ---- the same solve for nb <= 16 right-hand sides in lockstep
 bool coarse_gcr_batch_ok(const Level &L, int restart, int nb);
 size_t coarse_gcr_batch_part_bytes(dwf_ctx *c);
@@ -153,9 +153,10 @@ void coarse_gcr_tc(dwf_ctx *c, const Level &L, float2 *x, const float2 *b, int n
 void build_tc_images(dwf_ctx *c, Level &L);
 // throws DWF_ETIMEOUT when a tensor-core solve since the last check gave up a bounded wait
 void check_tc_timeout(dwf_ctx *c);
+// max_ctas: CTAs of the cooperative grid at most (several solves at once share the SMs)
 template <typename R>
 void coarse_gcr_fused(dwf_ctx *c, const Level &L, C<R> *x, const C<R> *b, C<R> *r, C<R> *Z, C<R> *W, double2 *part,
-                      int *iters, double tol, int maxiter, int restart);
+                      int *iters, double tol, int maxiter, int restart, int max_ctas);
 
 template <typename T> void norm2_b(dwf_ctx *c, BatchScratch &bs, int base, int stride, const T *x, int64_t n, int nrhs);
 template <typename T>
