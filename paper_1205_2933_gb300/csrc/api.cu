@@ -127,6 +127,8 @@ dwf_status create_one(dwf_ctx **out, const int dims[4], int Ls, double M5, doubl
         DWF_CUDA(cudaMallocHost((void **)&c->hscal, sizeof(double) * dwf::NSCALAR));
         c->red_part.alloc(sizeof(double2) * 1024 * 8);
         c->red_count.alloc(sizeof(unsigned));
+        c->dn_count.alloc(sizeof(unsigned) * dwf::DN_COUNTERS);
+        DWF_CUDA(cudaMemsetAsync(c->dn_count.p, 0, c->dn_count.bytes, c->stream));
         DWF_CUDA(cudaMemsetAsync(c->red_count.p, 0, sizeof(unsigned), c->stream));
         DWF_CUDA(cudaStreamSynchronize(c->stream));
         return DWF_OK;

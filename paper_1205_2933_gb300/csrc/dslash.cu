@@ -12,6 +12,7 @@
 // Spin projection: see spin.cuh.
 #include <cstdlib>
 
+#include "dslash_norm.cuh"
 #include "spin.cuh"
 
 namespace dwf {
@@ -59,10 +60,14 @@ __device__ __forceinline__ void hop_row(C<R> acc[12], const C<R> *__restrict__ p
 // instructions per 5D site, 3.0 ms of the pipe at 16^3 x 32 x 16.  With the
 // complex multiply-add as four fused instructions 3.37 ms; as six 4.66 ms.
 // 168 registers and 3 CTAs per SM instead of 128 and 4 measured the same.
-template <typename R, bool DAG, bool SHFL, int LS, int MINB>
+// EPI 0 .. 4: the epilogues of the paired FP32 kernel (dslash_pair.cuh), here
+// for FP64: nothing, |out|^2, z - a D^+ in, z - D in, D in + a z (EPI > 0 runs
+// whole warps: blockDim.x a multiple of 32, no early exit before the norms).
+template <typename R, bool DAG, bool SHFL, int LS, int MINB, int EPI>
 __global__ void __launch_bounds__(128, MINB)
 dslash_kernel(C<R> *__restrict__ out, const C<R> *__restrict__ in, const C<R> *__restrict__ U, Geom g, R diag, R mf,
-              int spb, int64_t field) {
+              int spb, int64_t field, NormOut nout, ZUpdateT<R> zu) {
+    constexpr bool NORM = EPI == 1 || EPI == 2 || EPI == 4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C<R> *sU = reinterpret_cast<C<R> *>(smem_raw);               // [spb][8][10] (9 used)
     int *sN = reinterpret_cast<int *>(sU + (size_t)spb * 80);       // [spb][8]
@@ -95,14 +100,20 @@ dslash_kernel(C<R> *__restrict__ out, const C<R> *__restrict__ in, const C<R> *_
             sN[ls * 8 + k] = nb;
         }
     }
+    pdl_wait();  // the links are constant; fields and scalar slots are not
     __syncthreads();
     const int ls = threadIdx.x / Ls;
     const int s = threadIdx.x - ls * Ls;
     const int site = site0 + ls;
     const bool active = (ls < spb) && (site < V);
-    if (!SHFL && !active) return;
+    if (!SHFL && !NORM && !active) return;
     const int row = 12 * Ls;
     C<R> acc[12], self[12];
+    if (EPI >= 2 && active) {  // the second field, into L2 ahead of its use
+        const C<R> *zp = zu.zin + rhs_off + (size_t)site * row + s;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(zp + k * Ls));
+    }
     if (active) {
         const C<R> *p = in + (size_t)site * row + s;
 #pragma unroll
@@ -130,8 +141,8 @@ dslash_kernel(C<R> *__restrict__ out, const C<R> *__restrict__ in, const C<R> *_
             dn[k].x = __shfl_sync(0xffffffffu, self[dn_lo + k].x, ldn);
             dn[k].y = __shfl_sync(0xffffffffu, self[dn_lo + k].y, ldn);
         }
-        if (!active) return;
-    } else {
+        if (!NORM && !active) return;
+    } else if (active) {
         const C<R> *p = in + (size_t)site * row;
         const int sp = (s == Ls - 1) ? 0 : s + 1;
         const int sm = (s == 0) ? Ls - 1 : s - 1;
@@ -141,31 +152,64 @@ dslash_kernel(C<R> *__restrict__ out, const C<R> *__restrict__ in, const C<R> *_
             dn[k] = p[(dn_lo + k) * Ls + sm];
         }
     }
+    R nrm = 0;
+    if (!NORM || active) {
 #pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k] = diag * self[k];
+        for (int k = 0; k < 12; ++k) acc[k] = diag * self[k];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        acc[up_lo + k] = acc[up_lo + k] + cp * up[k];
-        acc[dn_lo + k] = acc[dn_lo + k] + cm * dn[k];
+        for (int k = 0; k < 6; ++k) {
+            acc[up_lo + k] = acc[up_lo + k] + cp * up[k];
+            acc[dn_lo + k] = acc[dn_lo + k] + cm * dn[k];
+        }
+        const C<R> *sUs = sU + ls * 80;
+        const int *sNs = sN + ls * 8;
+        const int fs = DAG ? +1 : -1;  // sig of the forward hops
+        hop_row<0, false, R, LS>(acc, in + (size_t)sNs[0] * row + s, Ls, sUs + 0 * 10, fs);
+        hop_row<0, true, R, LS>(acc, in + (size_t)sNs[4] * row + s, Ls, sUs + 4 * 10, -fs);
+        hop_row<1, false, R, LS>(acc, in + (size_t)sNs[1] * row + s, Ls, sUs + 1 * 10, fs);
+        hop_row<1, true, R, LS>(acc, in + (size_t)sNs[5] * row + s, Ls, sUs + 5 * 10, -fs);
+        hop_row<2, false, R, LS>(acc, in + (size_t)sNs[2] * row + s, Ls, sUs + 2 * 10, fs);
+        hop_row<2, true, R, LS>(acc, in + (size_t)sNs[6] * row + s, Ls, sUs + 6 * 10, -fs);
+        hop_row<3, false, R, LS>(acc, in + (size_t)sNs[3] * row + s, Ls, sUs + 3 * 10, fs);
+        hop_row<3, true, R, LS>(acc, in + (size_t)sNs[7] * row + s, Ls, sUs + 7 * 10, -fs);
+        pdl_dependents();
+        C<R> *o = out + (size_t)site * row + s;
+        R a = R(1);
+        if (EPI == 2 || EPI == 4) {
+            const double ww = zu.ww[(size_t)blockIdx.y * zu.stride];
+            a = ww > 0.0 ? (R)(zu.zz[(size_t)blockIdx.y * zu.stride] / ww) : R(0);
+        }
+        const C<R> *zp = EPI >= 2 ? zu.zin + rhs_off + (size_t)site * row + s : nullptr;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            C<R> v = acc[k];
+            if (EPI == 2 || EPI == 3) {
+                const C<R> z = zp[k * Ls];
+                v.x = z.x - a * v.x;
+                v.y = z.y - a * v.y;
+            } else if (EPI == 4) {
+                const C<R> z = zp[k * Ls];
+                v.x += a * z.x;
+                v.y += a * z.y;
+            }
+            o[k * Ls] = v;
+            if (NORM) {
+                nrm += v.x * v.x;
+                nrm += v.y * v.y;
+            }
+        }
     }
-    const C<R> *sUs = sU + ls * 80;
-    const int *sNs = sN + ls * 8;
-    const int fs = DAG ? +1 : -1;  // sig of the forward hops
-    hop_row<0, false, R, LS>(acc, in + (size_t)sNs[0] * row + s, Ls, sUs + 0 * 10, fs);
-    hop_row<0, true, R, LS>(acc, in + (size_t)sNs[4] * row + s, Ls, sUs + 4 * 10, -fs);
-    hop_row<1, false, R, LS>(acc, in + (size_t)sNs[1] * row + s, Ls, sUs + 1 * 10, fs);
-    hop_row<1, true, R, LS>(acc, in + (size_t)sNs[5] * row + s, Ls, sUs + 5 * 10, -fs);
-    hop_row<2, false, R, LS>(acc, in + (size_t)sNs[2] * row + s, Ls, sUs + 2 * 10, fs);
-    hop_row<2, true, R, LS>(acc, in + (size_t)sNs[6] * row + s, Ls, sUs + 6 * 10, -fs);
-    hop_row<3, false, R, LS>(acc, in + (size_t)sNs[3] * row + s, Ls, sUs + 3 * 10, fs);
-    hop_row<3, true, R, LS>(acc, in + (size_t)sNs[7] * row + s, Ls, sUs + 7 * 10, -fs);
-    C<R> *o = out + (size_t)site * row + s;
+    if constexpr (NORM) {
+        __shared__ double sh[33];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) o[k * Ls] = acc[k];
+        for (int o = 16; o > 0; o >>= 1) nrm += __shfl_down_sync(0xffffffffu, nrm, o);
+        norm_epilogue(nout, blockIdx.y, (double)nrm, sh);
+    }
 }
 
-template <typename R>
-void launch(dwf_ctx *c, C<R> *out, const C<R> *in, const C<R> *U, bool dag, int nrhs) {
+template <typename R, int EPI>
+void launch(dwf_ctx *c, C<R> *out, const C<R> *in, const C<R> *U, bool dag, int nrhs, double *nslot = nullptr,
+            int nstride = 0, const ZUpdateT<R> *zu = nullptr) {
     const Geom &g = c->g;
     DWF_REQUIRE(g.V * g.Ls * 12 < (int64_t)1 << 31 && g.V < (int64_t)1 << 31, DWF_EINVAL,
                 "lattice too large for 32-bit element offsets of one field");
@@ -175,44 +219,59 @@ void launch(dwf_ctx *c, C<R> *out, const C<R> *in, const C<R> *U, bool dag, int 
     const int max_spb = (int)((46 * 1024) / per_site);
     if (spb > max_spb) spb = max_spb;
     const bool shfl = (32 % g.Ls) == 0;
+    // FP64: smaller CTAs while the grid has less than six of them per SM, so that
+    // the FP64 pipes finish together (256 CTAs of 128 threads leave every third
+    // of 152 SMs' pipes idle half of the time: the FP64 V-cycle at 8^4 x 8 takes
+    // 1.58 ms with them, 1.50 with 1024 of 32)
+    if (sizeof(R) == 8)
+        while (spb > 1 && spb / 2 * g.Ls >= 32 && (g.V + spb - 1) / spb * nrhs < 6 * (int64_t)c->sm_count) spb /= 2;
     int threads = spb * g.Ls;
-    if (shfl) threads = (threads + 31) / 32 * 32;  // whole warps for the shuffles
+    if (shfl || EPI > 0) threads = (threads + 31) / 32 * 32;  // whole warps for the shuffles
     dim3 grid((unsigned)((g.V + spb - 1) / spb), (unsigned)nrhs);
     size_t smem = (size_t)spb * per_site;
     int64_t field = g.V * g.Ls * 12;
     R diag = R(5.0 - c->M5), mf = R(c->mf);
+    const NormOut nout = nslot ? norm_out(c, grid, nrhs, nslot, nstride) : NormOut{};
+    const ZUpdateT<R> z = zu ? *zu : ZUpdateT<R>{};
     // register budget: 8 CTAs/SM (64 registers, small spills) or 6 (80);
     // DWF_DSLASH_MINB=6 selects the latter
     static const int minb = [] {
         const char *e = getenv("DWF_DSLASH_MINB");
         return (e && atoi(e) == 6) ? 6 : 8;
     }();
-#define DLM(D, S, L, M) dslash_kernel<R, D, S, L, M><<<grid, threads, smem, c->stream>>>(out, in, U, g, diag, mf, spb, field)
+#define DLM(D, S, L, M)                                                                                             \
+    launch_after(dslash_kernel<R, D, S, L, M, EPI>, grid, dim3(threads), smem, c->stream, out, in, U, g, diag, mf, spb, \
+                 field, nout, z)
 #define DL(D, S, L)                                          \
     do {                                                     \
         if constexpr (sizeof(R) == 8) DLM(D, S, L, 4);       \
         else if (minb == 6) DLM(D, S, L, 6);                 \
         else DLM(D, S, L, 8);                                \
     } while (0)
-    if (g.Ls == 16) {
-        if (dag) DL(true, true, 16); else DL(false, true, 16);
-    } else if (g.Ls == 8) {
-        if (dag) DL(true, true, 8); else DL(false, true, 8);
-    } else if (dag) {
-        if (shfl) DL(true, true, 0); else DL(true, false, 0);
-    } else {
-        if (shfl) DL(false, true, 0); else DL(false, false, 0);
-    }
+    // (EPI 2 is a D^+ kernel, 3 and 4 are D kernels; the others come in both)
+#define DLD(S, L)                                            \
+    do {                                                     \
+        if constexpr (EPI == 2) DL(true, S, L);              \
+        else if constexpr (EPI > 2) DL(false, S, L);         \
+        else if (dag) DL(true, S, L);                        \
+        else DL(false, S, L);                                \
+    } while (0)
+    if (g.Ls == 16) DLD(true, 16);
+    else if (g.Ls == 8) DLD(true, 8);
+    else if (shfl) DLD(true, 0);
+    else DLD(false, 0);
+#undef DLD
 #undef DLM
 #undef DL
     DWF_CHECK_LAUNCH();
+    if (nslot) norm_finish(c, nout, grid, nrhs);
 }
 
 }  // namespace
 
 void dslash(dwf_ctx *c, double2 *out, const double2 *in, bool dag, int nrhs) {
     ProfScope ps(c, K_DSLASH_F64, nrhs);
-    launch<double>(c, out, in, c->U64.as<double2>(), dag, nrhs);
+    launch<double, 0>(c, out, in, c->U64.as<double2>(), dag, nrhs);
     c->applies64 += nrhs;
 }
 
@@ -261,7 +320,7 @@ void dslash(dwf_ctx *c, float2 *out, const float2 *in, bool dag, int nrhs) {
         c->applies32 += nrhs;
         return;
     }
-    launch<float>(c, out, in, c->U32.as<float2>(), dag, nrhs);
+    launch<float, 0>(c, out, in, c->U32.as<float2>(), dag, nrhs);
     c->applies32 += nrhs;
 }
 
@@ -300,6 +359,40 @@ void dslash_zupdate(dwf_ctx *c, float2 *zout, const float2 *w, const float2 *zin
     double *s = c->scal.as<double>();
     dslash_pair_f32(c, zout, w, true, nrhs, pair_minb(), s + slot, stride, zin, s + izz, s + iww);
     c->applies32 += nrhs;
+}
+
+void dslash_norm(dwf_ctx *c, double2 *out, const double2 *in, bool dag, int nrhs, int slot, int stride) {
+    ProfScope ps(c, K_DSLASH_F64, nrhs);
+    launch<double, 1>(c, out, in, c->U64.as<double2>(), dag, nrhs, c->scal.as<double>() + slot, stride);
+    c->applies64 += nrhs;
+}
+
+void dslash_residual(dwf_ctx *c, double2 *res, const double2 *x, const double2 *b, int nrhs) {
+    DWF_REQUIRE(res != x && res != b, DWF_EINVAL, "residual: output must not alias an input");
+    ProfScope ps(c, K_DSLASH_F64, nrhs);
+    const ZUpdateT<double> zu{b, nullptr, nullptr, 0, 0};
+    launch<double, 3>(c, res, x, c->U64.as<double2>(), false, nrhs, nullptr, 0, &zu);
+    c->applies64 += nrhs;
+}
+
+void dslash_wupdate(dwf_ctx *c, double2 *wout, const double2 *z, const double2 *win, int nrhs, int slot, int stride,
+                    int inum, int iden) {
+    DWF_REQUIRE(wout != win && wout != z, DWF_EINVAL, "direction update: output must not alias an input");
+    ProfScope ps(c, K_DSLASH_F64, nrhs);
+    double *s = c->scal.as<double>();
+    const ZUpdateT<double> zu{win, s + inum, s + iden, stride, 1};
+    launch<double, 4>(c, wout, z, c->U64.as<double2>(), false, nrhs, s + slot, stride, &zu);
+    c->applies64 += nrhs;
+}
+
+void dslash_zupdate(dwf_ctx *c, double2 *zout, const double2 *w, const double2 *zin, int nrhs, int slot, int stride,
+                    int izz, int iww) {
+    DWF_REQUIRE(zout != zin && zout != w, DWF_EINVAL, "residual update: output must not alias an input");
+    ProfScope ps(c, K_DSLASH_F64, nrhs);
+    double *s = c->scal.as<double>();
+    const ZUpdateT<double> zu{zin, s + izz, s + iww, stride, 0};
+    launch<double, 2>(c, zout, w, c->U64.as<double2>(), true, nrhs, s + slot, stride, &zu);
+    c->applies64 += nrhs;
 }
 
 }  // namespace dwf

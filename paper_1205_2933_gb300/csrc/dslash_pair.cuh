@@ -20,8 +20,7 @@
 #include <cmath>
 #include <cstdint>
 
-#include "dwf_internal.cuh"
-#include "fastdiv.cuh"
+#include "dslash_norm.cuh"
 
 namespace dwf {
 
@@ -227,8 +226,7 @@ constexpr int PAIR_THREADS = 128;  // at most; 128 registers per thread
 // A CTA stages its sites' links once and applies the operator to rb
 // right-hand sides in turn (r = blockIdx.y * rb + 0 .. rb-1, below nrhs).
 // EPI 0: out = D in (or D^+ in).  EPI 1: also |out_r|^2 of every right-hand
-// side r: one FP64 partial per CTA (FP32 per thread) into npart;
-// norm_finish_kernel adds them in a fixed order into the scalar slots.
+// side r: one FP64 partial per CTA (FP32 per warp), see dslash_norm.cuh.
 // EPI 2: out = zu.zin - a D^+ in, and |out_r|^2 as with EPI 1.
 // EPI 3: out = zu.zin - D in (a residual b - D x), no norm.
 // EPI 4: out = D in + a zu.zin (CGNR's w = D p carried as D z + b w), and |out_r|^2.
@@ -236,8 +234,7 @@ constexpr int PAIR_THREADS = 128;  // at most; 128 registers per thread
 template <bool DAG, int LS, int EPI>
 __global__ void __launch_bounds__(PAIR_THREADS, 4)
 dslash_pair_kernel(float2 *__restrict__ out0, const float2 *__restrict__ in0, const float2 *__restrict__ U, Geom g,
-                   Brick bk, float diag, float mf, int64_t field, double *__restrict__ npart, ZUpdate zu, int nrhs,
-                   int rb) {
+                   Brick bk, float diag, float mf, int64_t field, NormOut nout, ZUpdate zu, int nrhs, int rb) {
     constexpr bool NORM = EPI == 1 || EPI == 2 || EPI == 4;
     constexpr int TPS = LS / 2;      // lanes per site
     constexpr int SPW = 32 / TPS;    // sites per warp
@@ -251,7 +248,6 @@ dslash_pair_kernel(float2 *__restrict__ out0, const float2 *__restrict__ in0, co
     const bool active = brick_site(bk, g, blockIdx.x, ls, x) && wl < SPW;
     if (!active) x[0] = x[1] = x[2] = x[3] = 0;  // idle lanes compute on site 0 and store nothing
     const int site = site_of(g, x);
-    pdl_dependents();  // the next kernel's prologue may run beside this grid's tail
     // the links of the CTA's sites: U_mu(x) and U_mu(x-mu), two stored rows, the
     // third rebuilt as conj(row0 x row1) (det U = 1), scaled by the hop
     // coefficient and duplicated into (re, re, im, im)
@@ -343,6 +339,7 @@ dslash_pair_kernel(float2 *__restrict__ out0, const float2 *__restrict__ in0, co
             hop2<3, false>(acc, pa, sLs + 3 * 10, fs);
             if (EPI >= 2) ldrow<LS>(pa, zu.zin + (size_t)rhs * (size_t)field + self_off);
             hop2<3, true>(acc, pb, sLs + 7 * 10, -fs);
+            if (rhs + 1 == r1) pdl_dependents();
             float2 *o = out + self_off;
             float a = 1.f;
             if (EPI == 2 || EPI == 4) {
@@ -365,39 +362,11 @@ dslash_pair_kernel(float2 *__restrict__ out0, const float2 *__restrict__ in0, co
             if (EPI >= 2 && rhs + 1 < r1) request_z(rhs + 1);
         }
         if (NORM) {
-            __shared__ double wsum[PAIR_THREADS / 32];
+            __shared__ double wsum[33];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) nrm += __shfl_down_sync(0xffffffffu, nrm, o);
-            const int warp = threadIdx.x >> 5;
-            if (lane == 0) wsum[warp] = (double)nrm;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                double t = 0;
-                for (int w = 0; w < (int)blockDim.x >> 5; ++w) t += wsum[w];
-                npart[(size_t)rhs * gridDim.x + blockIdx.x] = t;
-            }
-            __syncthreads();  // wsum is rewritten for the next right-hand side
+            norm_epilogue(nout, rhs, (double)nrm, wsum);
         }
-    }
-}
-
-// nslot[r * nstride] = sum of the nb CTA partials of right-hand side r = blockIdx.x (fixed order)
-__global__ void __launch_bounds__(1024) norm_finish_kernel(const double *__restrict__ npart, double *__restrict__ nslot,
-                                                           int nstride, int nb) {
-    __shared__ double red[32];
-    pdl_dependents();
-    pdl_wait();
-    const double *pr = npart + (size_t)blockIdx.x * nb;
-    double t = 0;
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) t += pr[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double u = 0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) u += red[w];
-        nslot[(size_t)blockIdx.x * nstride] = u;
     }
 }
 
@@ -428,16 +397,11 @@ void dslash_pair_ls(dwf_ctx *c, float2 *out, const float2 *in, bool dag, int nrh
     const int64_t field = g.V * g.Ls * 12;
     const float diag = (float)(5.0 - c->M5), mf = (float)c->mf;
     const float2 *U = c->U32.as<float2>();
-    double *npart = nullptr;
-    if (nslot) {
-        const size_t pb = sizeof(double) * (size_t)grid.x * nrhs;
-        if (c->dn_part.bytes < pb) c->dn_part.alloc(pb);
-        npart = c->dn_part.as<double>();
-    }
+    const NormOut nout = nslot ? norm_out(c, grid, nrhs, nslot, nstride) : NormOut{};
     const ZUpdate z = zu ? *zu : ZUpdate{nullptr, nullptr, nullptr, 0, 0};
 #define PL(D, E)                                                                                                  \
     launch_after(dslash_pair_kernel<D, LS, E>, grid, dim3(threads), smem, c->stream, out, in, U, g, bk, diag, mf, \
-                 field, npart, z, nrhs, rb)
+                 field, nout, z, nrhs, rb)
     if (zu && !nslot) PL(false, 3);
     else if (zu && zu->add) PL(false, 4);
     else if (zu) PL(true, 2);
@@ -447,10 +411,7 @@ void dslash_pair_ls(dwf_ctx *c, float2 *out, const float2 *in, bool dag, int nrh
     else PL(false, 0);
 #undef PL
     DWF_CHECK_LAUNCH();
-    if (nslot) {
-        launch_after(norm_finish_kernel, dim3(nrhs), dim3(1024), 0, c->stream, npart, nslot, nstride, (int)grid.x);
-        DWF_CHECK_LAUNCH();
-    }
+    if (nslot) norm_finish(c, nout, grid, nrhs);
 }
 
 }  // namespace dwf

@@ -97,7 +97,11 @@ void note_launches(unsigned long long n);  // kernels launched by a replayed gra
 // pdl_dependents (or ended), and runs up to its pdl_wait beside that kernel's
 // tail; pdl_wait returns when the kernel before has completed and its writes
 // are visible.  Every such kernel calls pdl_wait before it touches anything a
-// kernel writes, so completion stays in stream order.
+// kernel writes, so completion stays in stream order.  pdl_dependents comes
+// late in the kernels here: CTAs that start while the grid before still fills
+// most SMs settle unevenly on what is left, which a grid of one wave never
+// makes up (FP64 V-cycle at 8^4 x 8: 2.28 ms with the call first, 1.50 without
+// dependent launch, 1.43 with the call before the epilogue).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -206,13 +210,14 @@ inline Brick pick_brick(const Geom &g, int sites) {
 
 // The normal-equations residual update of CGNR, z <- z - a D^+ w, with
 // a = zz / ww of each right-hand side read from the scalar slots.
-struct ZUpdate {
-    const float2 *zin;  // the second field (not the output buffer)
+template <typename R> struct ZUpdateT {
+    const C<R> *zin;    // the second field (not the output buffer)
     const double *zz;   // numerator of a for right-hand side r at zz[r * stride]
     const double *ww;   // denominator of a at ww[r * stride]
     int stride;
     int add;            // 1: out = D in + a zin (EPI 4); 0: out = zin - a D^+ in (EPI 2)
 };
+using ZUpdate = ZUpdateT<float>;
 
 // fifth extents of the paired FP32 Dslash, and its sites per warp there
 inline bool dslash_pair_supported(int Ls) {
@@ -221,6 +226,8 @@ inline bool dslash_pair_supported(int Ls) {
         default: return false;
     }
 }
+
+constexpr int DN_COUNTERS = 256;  // right-hand sides whose norms a small Dslash grid may add itself
 
 // Device scalar slots used by solver kernels (coefficients stay on the GPU).
 constexpr int NSCALAR = 8192;
@@ -272,6 +279,7 @@ struct dwf_ctx {
     dwf::DevBuf red_part, red_count;
     // per-CTA partial sums of the Dslash's fused output norms
     dwf::DevBuf dn_part;
+    dwf::DevBuf dn_count;  // ... and the counters of small grids (zero between launches)
     dwf::MGState *mg = nullptr;
     // error word of the tensor-core coarse solves (device int, owned by the
     // context: the solves' scratch is freed before the word is read back)
@@ -322,17 +330,23 @@ void dslash(dwf_ctx *c, float2 *out, const float2 *in, bool dag, int nrhs);
 // FP32 D (or D^+) that also writes |out_r|^2 to the double slot slot + r*stride
 // (available when dslash_norm_fused(c))
 bool dslash_norm_fused(dwf_ctx *c);
+void dslash_norm(dwf_ctx *c, double2 *out, const double2 *in, bool dag, int nrhs, int slot, int stride);
 void dslash_norm(dwf_ctx *c, float2 *out, const float2 *in, bool dag, int nrhs, int slot, int stride);
-// res = b - D x on nrhs FP32 fields (res distinct from x and b; when dslash_norm_fused(c))
+// res = b - D x on nrhs fields (res distinct from x and b; FP32 when dslash_norm_fused(c), as the two below)
+void dslash_residual(dwf_ctx *c, double2 *res, const double2 *x, const double2 *b, int nrhs);
 void dslash_residual(dwf_ctx *c, float2 *res, const float2 *x, const float2 *b, int nrhs);
 // CGNR's w = D p carried without p: w_out = D z + b w_in for every right-hand
 // side r, b = scal[inum + r stride] / scal[iden + r stride], and |w_out|^2 into
 // scal[slot + r stride] (when dslash_norm_fused(c))
+void dslash_wupdate(dwf_ctx *c, double2 *wout, const double2 *z, const double2 *win, int nrhs, int slot, int stride,
+                    int inum, int iden);
 void dslash_wupdate(dwf_ctx *c, float2 *wout, const float2 *z, const float2 *win, int nrhs, int slot, int stride,
                     int inum, int iden);
 // CGNR's normal-equations residual update z_out = z_in - a D^+ w for every
 // right-hand side r, a = scal[izz + r stride] / scal[iww + r stride], and
 // |z_out|^2 into scal[slot + r stride] (available when dslash_norm_fused(c))
+void dslash_zupdate(dwf_ctx *c, double2 *zout, const double2 *w, const double2 *zin, int nrhs, int slot, int stride,
+                    int izz, int iww);
 void dslash_zupdate(dwf_ctx *c, float2 *zout, const float2 *w, const float2 *zin, int nrhs, int slot, int stride,
                     int izz, int iww);
 

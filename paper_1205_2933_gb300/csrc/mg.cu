@@ -629,6 +629,9 @@ template <typename R> class BatchRunner {
 
     int64_t n(int l) const { return mg.lev[l].lg.nelem; }
 
+    // whether the Dslash has its fused epilogues: FP64 always, FP32 where the paired kernel runs
+    bool fused_ok() const { return sizeof(R) == 8 || dslash_norm_fused(c); }
+
     T *wsb(int l, int i) {
         auto &v = mg.wsb[l];
         if ((int)v.size() <= i) v.resize(i + 1);
@@ -705,12 +708,15 @@ template <typename R> class BatchRunner {
                 return false;
             }
             const size_t need = sizeof(T) * (size_t)n(0) * nr * (size_t)(nu + 1);
-            size_t fr = 0, tot = 0;
-            DWF_CUDA(cudaMemGetInfo(&fr, &tot));
             const auto &v = mg.wsb[0];
             bool held = (int)v.size() >= 100 + nu;
             for (int j = 0; held && j < nu; ++j) held = v[100 + j].bytes >= need / (nu + 1);
-            hist_ok_ = held || (double)need < 0.5 * (double)fr;
+            if (!held) {  // (the query costs tens of microseconds)
+                size_t fr = 0, tot = 0;
+                DWF_CUDA(cudaMemGetInfo(&fr, &tot));
+                held = (double)need < 0.5 * (double)fr;
+            }
+            hist_ok_ = held;
             hist_nu_ = nu;
         }
         return hist_ok_;
@@ -722,11 +728,10 @@ template <typename R> class BatchRunner {
             if (!accumulate) bzero<T>(c, x, NT);
             return;
         }
-        // the FP32 Dslash can produce the norms of its outputs in its epilogue
-        bool fused = false;
-        if constexpr (std::is_same<R, float>::value) fused = dslash_norm_fused(c);
+        // the Dslash can produce the norms of its outputs in its epilogue
+        const bool fused = fused_ok();
         T *w = wsb(0, 3);
-        if constexpr (std::is_same<R, float>::value) {
+        {
             if (fused && accumulate && rtol <= 0.0 && iters <= 32 && keep_history(iters)) {
                 // The smoother's form when its residuals z_0 .. z_{nu-1} fit in
                 // memory: no direction p and no per-iteration solution update.
@@ -806,8 +811,7 @@ template <typename R> class BatchRunner {
         int izz = 0, inew = 1;
         const int iww = 2;
         auto dnorm = [&](T *out, const T *in, bool dag, int slot) {
-            if constexpr (std::is_same<R, float>::value)
-                if (fused) return dslash_norm(c, out, in, dag, nr, SB + slot, SS);
+            if (fused) return dslash_norm(c, out, in, dag, nr, SB + slot, SS);
             dslash(c, out, in, dag, nr);
             norm2_b<T>(c, mg.bscratch, SB + slot, SS, out, N, nr);
         };
@@ -821,7 +825,7 @@ template <typename R> class BatchRunner {
             read_block(sv);
             for (int q = 0; q < nr; ++q) r0[q] = std::sqrt(sv[(size_t)q * SS + irr]);
         }
-        if constexpr (std::is_same<R, float>::value) {
+        {
             if (fused && !(accumulate && rtol > 0.0)) {
                 // r itself is never needed: the normal-equations residual
                 // z = D^+ r follows its own recursion z <- z - a D^+ w (the
@@ -1126,12 +1130,9 @@ template <typename R> class BatchRunner {
         coarse_solves(x2, b2, Nc);
         prolong_batch<R>(c, L, x, x2, one.Q(0), nr, false);
         if (mg.p.nu_post > 0) {
-            bool fused = false;
-            if constexpr (std::is_same<R, float>::value) {
-                fused = dslash_norm_fused(c);
-                if (fused) dslash_residual(c, res, x, b, nr);  // res = b - A x in the Dslash epilogue
-            }
-            if (!fused) {
+            if (fused_ok()) {
+                dslash_residual(c, res, x, b, nr);  // res = b - A x in the Dslash epilogue
+            } else {
                 dslash(c, res, x, false, nr);
                 cxpay<T>(c, res, make_double2(-1.0, 0.0), b, NT);  // res = b - A x
             }
@@ -1470,13 +1471,14 @@ bool batch_on() {
     return on;
 }
 
-// The batched path covers FP32 V-cycles on two levels with nu_1 = 0, one
-// right-hand side included (its smoother then needs 2 launches per step instead
-// of 6: a V-cycle at 8^3 x 16 x 16 in 1.07 ms instead of 1.50); an FP16 basis copy is used only
-// by the one-at-a-time V-cycle.  DWF_BATCH=0 in the environment turns it off.
+// The batched path covers V-cycles on two levels with nu_1 = 0, one right-hand
+// side included (its smoother then needs 2 launches per step instead of 6: a
+// FP32 V-cycle at 8^3 x 16 x 16 in 1.07 ms instead of 1.50; an FP64 one at
+// 8^4 x 8 in 1.43 ms instead of 1.65), FP64 always one at a time.  An FP16 basis copy is used only by
+// the other V-cycle.  DWF_BATCH=0 in the environment turns it off.
 template <typename R> bool batch_eligible(const MGState &mg, int nrhs) {
-    return std::is_same<R, float>::value && (nrhs > 1 || !mg.lev[0].Q16.p) && batch_on() && mg.nlevels == 2 &&
-           mg.p.nu_pre == 0 && mg.p.outer_restart <= 32 && mg.p.coarsen == 0;
+    return (nrhs > 1 || !mg.lev[0].Q16.p) && batch_on() && mg.nlevels == 2 && mg.p.nu_pre == 0 &&
+           mg.p.outer_restart <= 32 && mg.p.coarsen == 0;
 }
 
 // Right-hand sides per batch: at most 32, and no more than the free device
@@ -1502,9 +1504,11 @@ template <typename R> int batch_width(const MGState &mg, int nrhs, bool solve) {
             for (int i = 0; i < 2; ++i) g += std::max(0.0, (double)N * nb * sizeof(double2) - held(mg.wsb64, i));
         return g;
     };
+    const int most = std::is_same<R, double>::value ? 1 : std::min(32, nrhs);
+    if (growth(most) == 0.0) return most;  // everything is held: no need to ask for the free memory
     size_t fr = 0, tot = 0;
     DWF_CUDA(cudaMemGetInfo(&fr, &tot));
-    int nb = std::min(32, nrhs);
+    int nb = most;
     while (nb >= 1 && growth(nb) > 0.9 * (double)fr) --nb;
     return nb;  // 0: not even one
 }
@@ -1536,10 +1540,10 @@ dwf_status solve_t(dwf_ctx *c, MGState &mg, double2 *b, double2 *x, double tol, 
     // the width of the batches (0: one at a time without the batched path)
     auto fitting = [&] {
         const int w = batch_width<R>(mg, nrhs, true);
-        return w > 1 || nrhs == 1 ? w : 0;
+        return w > 1 || nrhs == 1 || std::is_same<R, double>::value ? w : 0;
     };
     int width = batch_eligible<R>(mg, nrhs) ? fitting() : 0;
-    if (batch_eligible<R>(mg, nrhs) && width < std::min(nrhs, 32) && !mg.wsb[0].empty()) {
+    if (std::is_same<R, float>::value && batch_eligible<R>(mg, nrhs) && width < std::min(nrhs, 32) && !mg.wsb[0].empty()) {
         // memory-bound: the workspaces another width left (e.g. the setup's
         // relaxation of all start vectors) give way to the solve's own
         for (int l = 0; l < MAX_LEVELS; ++l) mg.wsb[l].clear();
@@ -1798,7 +1802,7 @@ template <typename R> void coarse_solve_t(dwf_ctx *c, MGState &mg, int level, vo
 template <typename R> void vcycle_t(dwf_ctx *c, MGState &mg, double2 *x, const double2 *b, int nrhs) {
     const int64_t N = mg.lev[0].lg.nelem;
     int width = batch_eligible<R>(mg, nrhs) ? batch_width<R>(mg, nrhs, false) : 0;
-    if (width == 1 && nrhs > 1) width = 0;
+    if (width == 1 && nrhs > 1 && std::is_same<R, float>::value) width = 0;
     if (width > 0) {
         for (int r0 = 0; r0 < nrhs; r0 += width) {
             const int nb = std::min(width, nrhs - r0);
