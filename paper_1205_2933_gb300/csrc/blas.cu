@@ -3,7 +3,7 @@
 // and the last CTA to finish (atomic ticket) adds the partials in a fixed
 // order and stores the result in a device scalar slot, so that solver
 // coefficients can stay on the GPU.
-#include "dwf_internal.cuh"
+#include "reduce.cuh"
 
 namespace dwf {
 
@@ -11,56 +11,6 @@ namespace {
 
 constexpr int RED_THREADS = 256;
 constexpr int RED_MAX_BLOCKS = 1024;
-
-__device__ __forceinline__ double2 to_d(double2 a) { return a; }
-__device__ __forceinline__ double2 to_d(float2 a) { return make_double2(a.x, a.y); }
-
-__device__ __forceinline__ double2 block_sum(double2 v, double2 *sh) {
-    for (int o = 16; o > 0; o >>= 1) {
-        v.x += __shfl_down_sync(0xffffffffu, v.x, o);
-        v.y += __shfl_down_sync(0xffffffffu, v.y, o);
-    }
-    int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) sh[w] = v;
-    __syncthreads();
-    int nw = (blockDim.x + 31) >> 5;
-    v = (threadIdx.x < nw) ? sh[threadIdx.x] : make_double2(0, 0);
-    if (w == 0)
-        for (int o = 16; o > 0; o >>= 1) {
-            v.x += __shfl_down_sync(0xffffffffu, v.x, o);
-            v.y += __shfl_down_sync(0xffffffffu, v.y, o);
-        }
-    __syncthreads();
-    return v;  // valid in thread 0
-}
-
-// finish: last CTA reduces the partials; writes out[0] (and out[1] for complex)
-__device__ void finish(double2 mine, double2 *part, unsigned *count, double *out, bool complex_result) {
-    __shared__ double2 sh[32];
-    __shared__ bool last;
-    double2 t = block_sum(mine, sh);
-    if (threadIdx.x == 0) {
-        part[blockIdx.x] = t;
-        __threadfence();
-        unsigned ticket = atomicAdd(count, 1u);
-        last = (ticket == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    double2 v = make_double2(0, 0);
-    for (int i = threadIdx.x; i < gridDim.x; i += blockDim.x) {
-        const volatile double *pp = reinterpret_cast<const volatile double *>(&part[i]);
-        v.x += pp[0];
-        v.y += pp[1];
-    }
-    v = block_sum(v, sh);
-    if (threadIdx.x == 0) {
-        out[0] = v.x;
-        if (complex_result) out[1] = v.y;
-        *count = 0u;
-    }
-}
 
 // Per-thread partial sums in the storage precision (FP32 FMAs for FP32
 // fields), combined across threads and CTAs in FP64.
@@ -70,7 +20,7 @@ template <> struct Acc<float2> { using type = float; };
 
 template <typename TX, typename TY>
 __global__ void __launch_bounds__(RED_THREADS) dot_kernel(const TX *__restrict__ x, const TY *__restrict__ y, int64_t n,
-                                                          double2 *part, unsigned *count, double *out) {
+                                                          double *part, unsigned *count, double *out) {
     using A = typename Acc<TX>::type;
     A ar = 0, ai = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -81,11 +31,12 @@ __global__ void __launch_bounds__(RED_THREADS) dot_kernel(const TX *__restrict__
         ar += (A)u.y * (A)v.y;
         ai -= (A)u.y * (A)v.x;
     }
-    finish(make_double2((double)ar, (double)ai), part, count, out, true);
+    const double m[2] = {(double)ar, (double)ai};
+    grid_sums<2>(m, part, count, out, 2);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(RED_THREADS) norm2_kernel(const T *__restrict__ x, int64_t n, double2 *part,
+__global__ void __launch_bounds__(RED_THREADS) norm2_kernel(const T *__restrict__ x, int64_t n, double *part,
                                                             unsigned *count, double *out) {
     using A = typename Acc<T>::type;
     A a = 0;
@@ -94,7 +45,8 @@ __global__ void __launch_bounds__(RED_THREADS) norm2_kernel(const T *__restrict_
         a += (A)u.x * (A)u.x;
         a += (A)u.y * (A)u.y;
     }
-    finish(make_double2((double)a, 0.0), part, count, out, false);
+    const double m[1] = {(double)a};
+    grid_sums<1>(m, part, count, out, 1);
 }
 
 // out[2j], out[2j+1] = <V_j, w> for j < K: w is read once for K vectors.
@@ -104,7 +56,7 @@ template <typename T, int K> struct MultiDotArgs {
 
 template <typename T, int K>
 __global__ void __launch_bounds__(RED_THREADS) multidot_kernel(MultiDotArgs<T, K> a, const T *__restrict__ w, int64_t n,
-                                                               double2 *part, unsigned *count, double *out) {
+                                                               double *part, unsigned *count, double *out) {
     using A = typename Acc<T>::type;
     A ar[K], ai[K];
 #pragma unroll
@@ -120,34 +72,13 @@ __global__ void __launch_bounds__(RED_THREADS) multidot_kernel(MultiDotArgs<T, K
             ai[j] -= (A)u.y * (A)y.x;
         }
     }
-    __shared__ double2 sh[32];
-    __shared__ bool last;
+    double m[2 * K];
+#pragma unroll
     for (int j = 0; j < K; ++j) {
-        double2 t = block_sum(make_double2((double)ar[j], (double)ai[j]), sh);
-        if (threadIdx.x == 0) part[(size_t)j * gridDim.x + blockIdx.x] = t;
+        m[2 * j] = (double)ar[j];
+        m[2 * j + 1] = (double)ai[j];
     }
-    if (threadIdx.x == 0) {
-        __threadfence();
-        unsigned ticket = atomicAdd(count, 1u);
-        last = (ticket == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    for (int j = 0; j < K; ++j) {
-        double2 v = make_double2(0, 0);
-        for (int i = threadIdx.x; i < gridDim.x; i += blockDim.x) {
-            const volatile double *pp = reinterpret_cast<const volatile double *>(&part[(size_t)j * gridDim.x + i]);
-            v.x += pp[0];
-            v.y += pp[1];
-        }
-        v = block_sum(v, sh);
-        if (threadIdx.x == 0) {
-            out[2 * j] = v.x;
-            out[2 * j + 1] = v.y;
-        }
-    }
-    if (threadIdx.x == 0) *count = 0u;
+    grid_sums<2 * K>(m, part, count, out, 2 * K);
 }
 
 template <typename T>
@@ -162,8 +93,10 @@ __global__ void copy_kernel(TO *__restrict__ out, const TI *__restrict__ in, int
         out[i] = cvt<TO, TI>(in[i]);
 }
 
+// at least four elements per thread: every CTA ends with a ticket on one address
 unsigned red_blocks(dwf_ctx *c, int64_t n) {
-    int64_t b = (n + RED_THREADS - 1) / RED_THREADS;
+    int64_t b = std::max<int64_t>((n + 4 * RED_THREADS - 1) / (4 * RED_THREADS),
+                                  std::min<int64_t>((n + RED_THREADS - 1) / RED_THREADS, c->sm_count));
     int64_t cap = std::min<int64_t>(RED_MAX_BLOCKS, (int64_t)c->sm_count * 6);
     return (unsigned)std::max<int64_t>(1, std::min(b, cap));
 }
@@ -188,13 +121,13 @@ template <typename TO, typename TI> void bcopy(dwf_ctx *c, TO *out, const TI *in
 
 template <typename TX, typename TY> void bdot(dwf_ctx *c, int slot, const TX *x, const TY *y, int64_t n) {
     dot_kernel<TX, TY><<<red_blocks(c, n), RED_THREADS, 0, c->stream>>>(
-        x, y, n, c->red_part.as<double2>(), c->red_count.as<unsigned>(), c->scal.as<double>() + slot);
+        x, y, n, c->red_part.as<double>(), c->red_count.as<unsigned>(), c->scal.as<double>() + slot);
     DWF_CHECK_LAUNCH();
 }
 
 template <typename T> void bnorm2(dwf_ctx *c, int slot, const T *x, int64_t n) {
     norm2_kernel<T><<<red_blocks(c, n), RED_THREADS, 0, c->stream>>>(
-        x, n, c->red_part.as<double2>(), c->red_count.as<unsigned>(), c->scal.as<double>() + slot);
+        x, n, c->red_part.as<double>(), c->red_count.as<unsigned>(), c->scal.as<double>() + slot);
     DWF_CHECK_LAUNCH();
 }
 
@@ -250,7 +183,7 @@ template <typename T> void bmultidot(dwf_ctx *c, int slot, T *const *V, int k, c
     {                                                                                                    \
         MultiDotArgs<T, K> a;                                                                            \
         for (int j = 0; j < K; ++j) a.v[j] = V[j0 + j];                                                  \
-        multidot_kernel<T, K><<<nb, RED_THREADS, 0, c->stream>>>(a, w, n, c->red_part.as<double2>(),     \
+        multidot_kernel<T, K><<<nb, RED_THREADS, 0, c->stream>>>(a, w, n, c->red_part.as<double>(),     \
                                                                  c->red_count.as<unsigned>(),            \
                                                                  c->scal.as<double>() + slot + 2 * j0);  \
     }

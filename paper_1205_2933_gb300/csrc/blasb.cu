@@ -3,6 +3,7 @@
 // coefficients, read from device memory (scalar slots or coefficient
 // arrays), and its own deterministic FP64-accumulated reductions.
 #include "mg.cuh"
+#include "reduce.cuh"
 
 namespace dwf {
 
@@ -14,74 +15,23 @@ template <typename T> struct RealB;
 template <> struct RealB<float2> { using type = float; };
 template <> struct RealB<double2> { using type = double; };
 
-__device__ __forceinline__ double2 bsum(double2 v, double2 *sh) {
-    for (int o = 16; o > 0; o >>= 1) {
-        v.x += __shfl_down_sync(0xffffffffu, v.x, o);
-        v.y += __shfl_down_sync(0xffffffffu, v.y, o);
-    }
-    int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    if (l == 0) sh[w] = v;
-    __syncthreads();
-    v = (threadIdx.x < (blockDim.x + 31) / 32) ? sh[threadIdx.x] : make_double2(0, 0);
-    if (w == 0)
-        for (int o = 16; o > 0; o >>= 1) {
-            v.x += __shfl_down_sync(0xffffffffu, v.x, o);
-            v.y += __shfl_down_sync(0xffffffffu, v.y, o);
-        }
-    __syncthreads();
-    return v;
-}
-
-// K complex reductions per right-hand side: out[base + r*stride + 2j (+1)];
-// a real result (CPLX = false, K = 1) writes the single slot base + r*stride
-template <int K, bool CPLX = true>
-__device__ void finish_b(const double2 (&mine)[K], double2 *part, unsigned *count, double *s, int base, int stride) {
-    __shared__ double2 sh[32];
-    __shared__ bool last;
-    const int r = blockIdx.y, nb = gridDim.x;
-    double2 *pr = part + (size_t)r * K * nb;
-    for (int j = 0; j < K; ++j) {
-        double2 t = bsum(mine[j], sh);
-        if (threadIdx.x == 0) pr[(size_t)j * nb + blockIdx.x] = t;
-    }
-    if (threadIdx.x == 0) {
-        __threadfence();
-        unsigned ticket = atomicAdd(count + r, 1u);
-        last = (ticket == nb - 1);
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    for (int j = 0; j < K; ++j) {
-        double2 v = make_double2(0, 0);
-        for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-            const volatile double *pp = reinterpret_cast<const volatile double *>(&pr[(size_t)j * nb + i]);
-            v.x += pp[0];
-            v.y += pp[1];
-        }
-        v = bsum(v, sh);
-        if (threadIdx.x == 0) {
-            s[base + r * stride + 2 * j] = v.x;
-            if (CPLX) s[base + r * stride + 2 * j + 1] = v.y;
-        }
-    }
-    if (threadIdx.x == 0) count[r] = 0u;
-}
-
 // s[base + r*stride] = |x_r|^2
 template <typename T>
-__global__ void __launch_bounds__(BT) norm2_b_kernel(const T *__restrict__ x, int64_t n, double2 *part, unsigned *count,
+__global__ void __launch_bounds__(BT) norm2_b_kernel(const T *__restrict__ x, int64_t n, double *part, unsigned *count,
                                                      double *s, int base, int stride) {
     using A = typename RealB<T>::type;
     x += (size_t)blockIdx.y * n;
     A a = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        T u = x[i];
-        a += u.x * u.x;
-        a += u.y * u.y;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n / Pack<T>::N; i += (int64_t)gridDim.x * blockDim.x) {
+        const Pack<T> u = ldp(x, i);
+#pragma unroll
+        for (int e = 0; e < Pack<T>::N; ++e) {
+            a += u.e[e].x * u.e[e].x;
+            a += u.e[e].y * u.e[e].y;
+        }
     }
-    double2 m[1] = {make_double2((double)a, 0.0)};
-    finish_b<1, false>(m, part, count, s, base, stride);
+    const double m[1] = {(double)a};
+    grid_sums<1>(m, part + (size_t)blockIdx.y * gridDim.x, count + blockIdx.y, s + base + blockIdx.y * stride, 1);
 }
 
 // s[base + r*stride + 2j (+1)] = <V_j,r, w_r>, j < K (w read once)
@@ -90,28 +40,36 @@ template <typename T, int K> struct VArgs {
 };
 template <typename T, int K>
 __global__ void __launch_bounds__(BT) multidot_b_kernel(VArgs<T, K> va, const T *__restrict__ w, int64_t n,
-                                                        double2 *part, unsigned *count, double *s, int base,
+                                                        double *part, unsigned *count, double *s, int base,
                                                         int stride) {
     using A = typename RealB<T>::type;
     const size_t off = (size_t)blockIdx.y * n;
     A ar[K], ai[K];
 #pragma unroll
     for (int j = 0; j < K; ++j) ar[j] = ai[j] = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        T y = w[off + i];
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n / Pack<T>::N; i += (int64_t)gridDim.x * blockDim.x) {
+        const Pack<T> y = ldp(w + off, i);
+        Pack<T> u[K];
 #pragma unroll
-        for (int j = 0; j < K; ++j) {
-            T u = va.v[j][off + i];
-            ar[j] += u.x * y.x;
-            ai[j] += u.x * y.y;
-            ar[j] += u.y * y.y;
-            ai[j] -= u.y * y.x;
-        }
+        for (int j = 0; j < K; ++j) u[j] = ldp(va.v[j] + off, i);
+#pragma unroll
+        for (int j = 0; j < K; ++j)
+#pragma unroll
+            for (int e = 0; e < Pack<T>::N; ++e) {
+                ar[j] += u[j].e[e].x * y.e[e].x;
+                ai[j] += u[j].e[e].x * y.e[e].y;
+                ar[j] += u[j].e[e].y * y.e[e].y;
+                ai[j] -= u[j].e[e].y * y.e[e].x;
+            }
     }
-    double2 m[K];
+    double m[2 * K];
 #pragma unroll
-    for (int j = 0; j < K; ++j) m[j] = make_double2((double)ar[j], (double)ai[j]);
-    finish_b<K>(m, part, count, s, base, stride);
+    for (int j = 0; j < K; ++j) {
+        m[2 * j] = (double)ar[j];
+        m[2 * j + 1] = (double)ai[j];
+    }
+    grid_sums<2 * K>(m, part + (size_t)blockIdx.y * 2 * K * gridDim.x, count + blockIdx.y,
+                     s + base + blockIdx.y * stride, 2 * K);
 }
 
 // w_r += sgn * sum_j c_{r,j} V_j,r with c from slots s[base + r*stride + 2j]
@@ -131,17 +89,20 @@ __global__ void multiaxpy_b_kernel(T *__restrict__ w, MArgs<T> a, const double *
         ci[threadIdx.x] = (R)(sgn * s[base + r * stride + 2 * threadIdx.x + 1]);
     }
     __syncthreads();
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        T v = w[off + i];
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n / Pack<T>::N; i += (int64_t)gridDim.x * blockDim.x) {
+        Pack<T> v = ldp<T>(w + off, i);
 #pragma unroll 8
         for (int j = 0; j < a.k; ++j) {
-            T u = a.v[j][off + i];
-            v.x += cr[j] * u.x;
-            v.y += cr[j] * u.y;
-            v.x -= ci[j] * u.y;
-            v.y += ci[j] * u.x;
+            const Pack<T> u = ldp(a.v[j] + off, i);
+#pragma unroll
+            for (int e = 0; e < Pack<T>::N; ++e) {
+                v.e[e].x += cr[j] * u.e[e].x;
+                v.e[e].y += cr[j] * u.e[e].y;
+                v.e[e].x -= ci[j] * u.e[e].y;
+                v.e[e].y += ci[j] * u.e[e].x;
+            }
         }
-        w[off + i] = v;
+        stp(w + off, i, v);
     }
 }
 
@@ -258,22 +219,24 @@ __global__ void normalised_b_kernel(double2 *__restrict__ out, const T *__restri
     }
 }
 
-// w_r *= sc[r];  res_r -= al[r] * w_r   (GCR direction normalisation and residual update)
+// w_r *= scale[r];  res_r -= al[r] * w_r   (GCR direction normalisation and residual update)
 template <typename T>
-__global__ void gcr_wr_b_kernel(T *__restrict__ w, T *__restrict__ res, const double *__restrict__ sc,
-                                const double2 *__restrict__ al, int64_t n) {
+__global__ void gcr_wr_b_kernel(T *__restrict__ w, T *__restrict__ res, GcrStep step, int64_t n) {
     using R = typename RealB<T>::type;
     const int r = blockIdx.y;
     const size_t off = (size_t)r * n;
-    const R s = (R)sc[r], ar = (R)al[r].x, ai = (R)al[r].y;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        T wv = w[off + i], rv = res[off + i];
-        wv.x *= s;
-        wv.y *= s;
-        rv.x -= ar * wv.x - ai * wv.y;
-        rv.y -= ar * wv.y + ai * wv.x;
-        w[off + i] = wv;
-        res[off + i] = rv;
+    const R s = (R)step.scale[r], ar = (R)step.al[r].x, ai = (R)step.al[r].y;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n / Pack<T>::N; i += (int64_t)gridDim.x * blockDim.x) {
+        Pack<T> wv = ldp<T>(w + off, i), rv = ldp<T>(res + off, i);
+#pragma unroll
+        for (int e = 0; e < Pack<T>::N; ++e) {
+            wv.e[e].x *= s;
+            wv.e[e].y *= s;
+            rv.e[e].x -= ar * wv.e[e].x - ai * wv.e[e].y;
+            rv.e[e].y -= ar * wv.e[e].y + ai * wv.e[e].x;
+        }
+        stp(w + off, i, wv);
+        stp(res + off, i, rv);
     }
 }
 
@@ -289,17 +252,20 @@ __global__ void combo_b_kernel(T *__restrict__ x, MArgs<T> a, const double2 *__r
         ci[threadIdx.x] = (R)g[r * a.k + threadIdx.x].y;
     }
     __syncthreads();
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        T v = x[off + i];
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n / Pack<T>::N; i += (int64_t)gridDim.x * blockDim.x) {
+        Pack<T> v = ldp<T>(x + off, i);
 #pragma unroll 8
         for (int j = 0; j < a.k; ++j) {
-            T u = a.v[j][off + i];
-            v.x += cr[j] * u.x;
-            v.y += cr[j] * u.y;
-            v.x -= ci[j] * u.y;
-            v.y += ci[j] * u.x;
+            const Pack<T> u = ldp(a.v[j] + off, i);
+#pragma unroll
+            for (int e = 0; e < Pack<T>::N; ++e) {
+                v.e[e].x += cr[j] * u.e[e].x;
+                v.e[e].y += cr[j] * u.e[e].y;
+                v.e[e].x -= ci[j] * u.e[e].y;
+                v.e[e].y += ci[j] * u.e[e].x;
+            }
         }
-        x[off + i] = v;
+        stp(x + off, i, v);
     }
 }
 
@@ -313,29 +279,37 @@ __global__ void cg_combine_b_kernel(T *__restrict__ x, MArgs<T> a, const double 
                                     int zb, int wb, int64_t n) {
     using R = typename RealB<T>::type;
     __shared__ R gam[32];
+    __shared__ double al[32], be[32];
     const int r = blockIdx.y;
     const size_t off = (size_t)r * n;
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < a.k) {  // the divisions side by side, the recurrence by one thread
+        const int j = threadIdx.x;
         const double *sr = s + base + (size_t)r * stride;
+        const double zz = sr[zb + j], ww = sr[wb + j];
+        al[j] = ww > 0.0 ? zz / ww : 0.0;
+        be[j] = (j + 1 < a.k && zz > 0.0) ? sr[zb + j + 1] / zz : 0.0;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
         double g = 0.0;
         for (int j = a.k - 1; j >= 0; --j) {
-            const double zz = sr[zb + j], ww = sr[wb + j];
-            const double al = ww > 0.0 ? zz / ww : 0.0;
-            const double be = (j + 1 < a.k && zz > 0.0) ? sr[zb + j + 1] / zz : 0.0;
-            g = al + be * g;
+            g = al[j] + be[j] * g;
             gam[j] = (R)g;
         }
     }
     __syncthreads();
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        T v = x[off + i];
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n / Pack<T>::N; i += (int64_t)gridDim.x * blockDim.x) {
+        Pack<T> v = ldp<T>(x + off, i);
 #pragma unroll 8
         for (int j = 0; j < a.k; ++j) {
-            const T u = a.v[j][off + i];
-            v.x += gam[j] * u.x;
-            v.y += gam[j] * u.y;
+            const Pack<T> u = ldp(a.v[j] + off, i);
+#pragma unroll
+            for (int e = 0; e < Pack<T>::N; ++e) {
+                v.e[e].x += gam[j] * u.e[e].x;
+                v.e[e].y += gam[j] * u.e[e].y;
+            }
         }
-        x[off + i] = v;
+        stp(x + off, i, v);
     }
 }
 
@@ -355,49 +329,68 @@ __global__ void cg_chunk_b_kernel(T *__restrict__ x, T *__restrict__ p, MArgs<T>
                                   int64_t n) {
     using R = typename RealB<T>::type;
     __shared__ R G[33], P[33];
+    __shared__ double al[32], be[32];
     const int r = blockIdx.y;
     const size_t off = (size_t)r * n;
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < m) {  // the divisions side by side, the recurrences by one thread
+        const int t = threadIdx.x;
         const double *sr = s + base + (size_t)r * stride;
-        auto zz = [&](int t) { return sr[zb + (k0 + t) % rs]; };
-        auto ww = [&](int t) { return sr[wb + (k0 + t) % rs]; };
+        const double zt = sr[zb + (k0 + t) % rs], wt = sr[wb + (k0 + t) % rs];
+        al[t] = wt > 0.0 ? zt / wt : 0.0;
+        be[t] = ((t + 1 < m || next) && zt > 0.0) ? sr[zb + (k0 + t + 1) % rs] / zt : 0.0;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
         double g = 0.0, q = 1.0;
         if (next) P[m] = (R)1;
         for (int t = m - 1; t >= 0; --t) {
-            const double zt = zz(t), wt = ww(t);
-            const double al = wt > 0.0 ? zt / wt : 0.0;
-            const bool have_b = t + 1 < m || next;
-            const double be = (have_b && zt > 0.0) ? zz(t + 1) / zt : 0.0;
-            g = al + (t + 1 < m ? be * g : 0.0);
+            g = al[t] + (t + 1 < m ? be[t] * g : 0.0);
             G[t] = (R)g;
             if (next) {
-                q *= be;
+                q *= be[t];
                 P[t] = (R)q;
             }
         }
     }
     __syncthreads();
-    const int nz = next ? m : m - 1;  // z pointers: z_1 .. z_nz
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const T pv = p[off + i];
-        T xv = xinit ? T{0, 0} : x[off + i];
-        T pn = next ? T{P[0] * pv.x, P[0] * pv.y} : T{0, 0};
-        xv.x += G[0] * pv.x;
-        xv.y += G[0] * pv.y;
+    const R p0 = next ? P[0] : R(0);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n / Pack<T>::N; i += (int64_t)gridDim.x * blockDim.x) {
+        const Pack<T> pv = ldp<T>(p + off, i);
+        Pack<T> xv, pn;
+        if (xinit) {
+#pragma unroll
+            for (int e = 0; e < Pack<T>::N; ++e) xv.e[e] = T{0, 0};
+        } else {
+            xv = ldp<T>(x + off, i);
+        }
+#pragma unroll
+        for (int e = 0; e < Pack<T>::N; ++e) {
+            pn.e[e].x = p0 * pv.e[e].x;
+            pn.e[e].y = p0 * pv.e[e].y;
+            xv.e[e].x += G[0] * pv.e[e].x;
+            xv.e[e].y += G[0] * pv.e[e].y;
+        }
 #pragma unroll 8
-        for (int t = 1; t <= nz; ++t) {
-            const T u = z.v[t - 1][off + i];
-            if (t < m) {
-                xv.x += G[t] * u.x;
-                xv.y += G[t] * u.y;
-            }
-            if (next) {
-                pn.x += P[t] * u.x;
-                pn.y += P[t] * u.y;
+        for (int t = 1; t < m; ++t) {
+            const Pack<T> u = ldp(z.v[t - 1] + off, i);
+#pragma unroll
+            for (int e = 0; e < Pack<T>::N; ++e) {
+                xv.e[e].x += G[t] * u.e[e].x;
+                xv.e[e].y += G[t] * u.e[e].y;
+                pn.e[e].x += P[t] * u.e[e].x;  // (not used by the last chunk)
+                pn.e[e].y += P[t] * u.e[e].y;
             }
         }
-        x[off + i] = xv;
-        if (next) p[off + i] = pn;
+        stp(x + off, i, xv);
+        if (next) {
+            const Pack<T> u = ldp(z.v[m - 1] + off, i);
+#pragma unroll
+            for (int e = 0; e < Pack<T>::N; ++e) {
+                pn.e[e].x += u.e[e].x;  // P_m = 1
+                pn.e[e].y += u.e[e].y;
+            }
+            stp(p + off, i, pn);
+        }
     }
 }
 
@@ -416,11 +409,22 @@ __global__ void cg_redirect_kernel(T *__restrict__ p, const T *__restrict__ zt, 
     }
 }
 
-dim3 grid_b(dwf_ctx *c, int64_t n, int nrhs, int cap_per_sm) {
-    int64_t b = (n + BT - 1) / BT;
+// CTAs per right-hand side: one pass of 16 bytes per thread up to cap_per_sm
+// CTAs per SM over all right-hand sides
+template <typename T> dim3 grid_b(dwf_ctx *c, int64_t n, int nrhs, int cap_per_sm) {
+    int64_t b = (n + BT * Pack<T>::N - 1) / (BT * Pack<T>::N);
     int64_t cap = std::max<int64_t>(1, (int64_t)c->sm_count * cap_per_sm / std::max(1, nrhs));
     cap = std::min<int64_t>(cap, 1024);  // partial-sum buffers hold 1024 blocks per value
     return dim3((unsigned)std::max<int64_t>(1, std::min(b, cap)), (unsigned)nrhs);
+}
+
+// ... and of a reduction: fewer CTAs, at least four passes each, since every one
+// of them ends with a ticket on one address
+template <typename T> dim3 grid_r(dwf_ctx *c, int64_t n, int nrhs) {
+    dim3 g = grid_b<T>(c, n, nrhs, 8);
+    const int64_t b = (n + BT * Pack<T>::N * 4 - 1) / (BT * Pack<T>::N * 4);
+    g.x = (unsigned)std::max<int64_t>(1, std::min<int64_t>(g.x, std::max<int64_t>(b, c->sm_count / nrhs)));
+    return g;
 }
 
 }  // namespace
@@ -436,22 +440,22 @@ void BatchScratch::ensure(int nrhs) {
 }
 
 template <typename T> void norm2_b(dwf_ctx *c, BatchScratch &bs, int base, int stride, const T *x, int64_t n, int nrhs) {
-    dim3 g = grid_b(c, n, nrhs, 8);
-    norm2_b_kernel<T><<<g, BT, 0, c->stream>>>(x, n, bs.part.as<double2>(), bs.count.as<unsigned>(), c->scal.as<double>(),
+    dim3 g = grid_r<T>(c, n, nrhs);
+    norm2_b_kernel<T><<<g, BT, 0, c->stream>>>(x, n, bs.part.as<double>(), bs.count.as<unsigned>(), c->scal.as<double>(),
                                                base, stride);
     DWF_CHECK_LAUNCH();
 }
 
 template <typename T>
 void multidot_b(dwf_ctx *c, BatchScratch &bs, int base, int stride, T *const *V, int k, const T *w, int64_t n, int nrhs) {
-    dim3 g = grid_b(c, n, nrhs, 8);
+    dim3 g = grid_r<T>(c, n, nrhs);
     for (int j0 = 0; j0 < k; j0 += 8) {
         int kk = std::min(8, k - j0);
 #define MDB(K)                                                                                              \
     {                                                                                                       \
         VArgs<T, K> a;                                                                                      \
         for (int j = 0; j < K; ++j) a.v[j] = V[j0 + j];                                                     \
-        multidot_b_kernel<T, K><<<g, BT, 0, c->stream>>>(a, w, n, bs.part.as<double2>(), bs.count.as<unsigned>(), \
+        multidot_b_kernel<T, K><<<g, BT, 0, c->stream>>>(a, w, n, bs.part.as<double>(), bs.count.as<unsigned>(), \
                                                          c->scal.as<double>(), base + 2 * j0, stride);      \
     }
         switch (kk) {
@@ -471,7 +475,7 @@ void multidot_b(dwf_ctx *c, BatchScratch &bs, int base, int stride, T *const *V,
 
 template <typename T>
 void multiaxpy_b(dwf_ctx *c, T *w, T *const *V, int k, int base, int stride, double sgn, int64_t n, int nrhs) {
-    dim3 g = grid_b(c, n, nrhs, 16);
+    dim3 g = grid_b<T>(c, n, nrhs, 16);
     for (int j0 = 0; j0 < k; j0 += 32) {
         MArgs<T> a;
         a.k = std::min(32, k - j0);
@@ -483,7 +487,7 @@ void multiaxpy_b(dwf_ctx *c, T *w, T *const *V, int k, int base, int stride, dou
 
 template <typename T>
 void cg_r_b(dwf_ctx *c, T *r, const T *rin, const T *w, int base, int stride, int izz, int iww, int64_t n, int nrhs) {
-    dim3 g = grid_b(c, n, nrhs, 16);
+    dim3 g = grid_b<T>(c, n, nrhs, 16);
     cg_r_b_kernel<T><<<g, BT, 0, c->stream>>>(r, rin, w, c->scal.as<double>(), base, stride, izz, iww, n);
     DWF_CHECK_LAUNCH();
 }
@@ -491,7 +495,7 @@ void cg_r_b(dwf_ctx *c, T *r, const T *rin, const T *w, int base, int stride, in
 template <typename T>
 void cg_px_b(dwf_ctx *c, T *x, T *pout, const T *pin, const T *z, int base, int stride, int izz, int iww, int inew,
              int64_t n, int nrhs, bool last, bool xinit) {
-    dim3 g = grid_b(c, n, nrhs, 16);
+    dim3 g = grid_b<T>(c, n, nrhs, 16);
     cg_px_b_kernel<T><<<g, BT, 0, c->stream>>>(x, pout, pin, z, c->scal.as<double>(), base, stride, izz, iww, inew,
                                                n, last ? 1 : 0, xinit ? 1 : 0);
     DWF_CHECK_LAUNCH();
@@ -502,7 +506,7 @@ void cg_pxd_b(dwf_ctx *c, T *x, T *pout, const T *pin, T *const *pend, int np, c
               int izz, int iww, int inew, int ia, int64_t n, int nrhs, int mode) {
     DWF_REQUIRE(mode >= 0 && mode <= 2 && np >= 0 && np <= CG_MAXDEFER && !(mode == 0 && np == CG_MAXDEFER),
                 DWF_EINVAL, "cg_pxd_b: mode or pending count");
-    dim3 g = grid_b(c, n, nrhs, 16);
+    dim3 g = grid_b<T>(c, n, nrhs, 16);
     Pending<T> pd{};
     for (int j = 0; j < np; ++j) pd.p[j] = pend[j];
     double *s = c->scal.as<double>();
@@ -520,22 +524,22 @@ void cg_pxd_b(dwf_ctx *c, T *x, T *pout, const T *pin, T *const *pend, int np, c
 
 template <typename T>
 void normalised_b(dwf_ctx *c, double2 *out, const T *x, int base, int stride, int64_t n, int nrhs) {
-    dim3 g = grid_b(c, n, nrhs, 16);
+    dim3 g = grid_b<T>(c, n, nrhs, 16);
     normalised_b_kernel<T><<<g, BT, 0, c->stream>>>(out, x, c->scal.as<double>(), base, stride, n);
     DWF_CHECK_LAUNCH();
 }
 
-template <typename T>
-void gcr_wr_b(dwf_ctx *c, T *w, T *res, const double *sc, const double2 *al, int64_t n, int nrhs) {
-    dim3 g = grid_b(c, n, nrhs, 16);
-    gcr_wr_b_kernel<T><<<g, BT, 0, c->stream>>>(w, res, sc, al, n);
+template <typename T> void gcr_wr_b(dwf_ctx *c, T *w, T *res, const GcrStep &step, int64_t n, int nrhs) {
+    DWF_REQUIRE(nrhs <= 32, DWF_EINVAL, "GCR step: at most 32 right-hand sides");
+    dim3 g = grid_b<T>(c, n, nrhs, 16);
+    gcr_wr_b_kernel<T><<<g, BT, 0, c->stream>>>(w, res, step, n);
     DWF_CHECK_LAUNCH();
 }
 
 template <typename T> void combo_b(dwf_ctx *c, T *x, T *const *V, int k, const double2 *g, int64_t n, int nrhs) {
     DWF_REQUIRE(k <= 32, DWF_EINVAL, "combo_b: at most 32 vectors");
     if (k == 0) return;
-    dim3 gr = grid_b(c, n, nrhs, 16);
+    dim3 gr = grid_b<T>(c, n, nrhs, 16);
     MArgs<T> a;
     a.k = k;
     for (int j = 0; j < k; ++j) a.v[j] = V[j];
@@ -546,7 +550,7 @@ template <typename T> void combo_b(dwf_ctx *c, T *x, T *const *V, int k, const d
 template <typename T>
 void cg_combine_b(dwf_ctx *c, T *x, T *const *Z, int k, int base, int stride, int zb, int wb, int64_t n, int nrhs) {
     DWF_REQUIRE(k >= 1 && k <= 32, DWF_EINVAL, "cg_combine_b: 1 to 32 stored residuals");
-    dim3 gr = grid_b(c, n, nrhs, 16);
+    dim3 gr = grid_b<T>(c, n, nrhs, 16);
     MArgs<T> a;
     a.k = k;
     for (int j = 0; j < k; ++j) a.v[j] = Z[j];
@@ -558,7 +562,7 @@ template <typename T>
 void cg_chunk_b(dwf_ctx *c, T *x, T *p, T *const *Z, int m, bool next, bool xinit, int base, int stride, int zb, int wb,
                 int k0, int rs, int64_t n, int nrhs) {
     DWF_REQUIRE(m >= 1 && m <= 32 && rs > m, DWF_EINVAL, "cg_chunk_b: 1 to 32 iterations, slot ring longer than that");
-    dim3 gr = grid_b(c, n, nrhs, 16);
+    dim3 gr = grid_b<T>(c, n, nrhs, 16);
     MArgs<T> a;
     a.k = next ? m : m - 1;
     for (int j = 0; j < a.k; ++j) a.v[j] = Z[j];
@@ -569,7 +573,7 @@ void cg_chunk_b(dwf_ctx *c, T *x, T *p, T *const *Z, int m, bool next, bool xini
 
 template <typename T>
 void cg_redirect(dwf_ctx *c, T *p, const T *zt, const T *z, int izt, int iz, int64_t n) {
-    cg_redirect_kernel<T><<<grid_b(c, n, 1, 16), BT, 0, c->stream>>>(p, zt, z, c->scal.as<double>(), izt, iz, n);
+    cg_redirect_kernel<T><<<grid_b<T>(c, n, 1, 16), BT, 0, c->stream>>>(p, zt, z, c->scal.as<double>(), izt, iz, n);
     DWF_CHECK_LAUNCH();
 }
 
@@ -587,7 +591,7 @@ void cg_redirect(dwf_ctx *c, T *p, const T *zt, const T *z, int izt, int iz, int
                                 int64_t, int);                                                                 \
     template void normalised_b<T>(dwf_ctx *, double2 *, const T *, int, int, int64_t, int);                   \
     template void cg_redirect<T>(dwf_ctx *, T *, const T *, const T *, int, int, int64_t);                   \
-    template void gcr_wr_b<T>(dwf_ctx *, T *, T *, const double *, const double2 *, int64_t, int);            \
+    template void gcr_wr_b<T>(dwf_ctx *, T *, T *, const GcrStep &, int64_t, int);                           \
     template void combo_b<T>(dwf_ctx *, T *, T *const *, int, const double2 *, int64_t, int);
 INSTB(float2)
 INSTB(double2)

@@ -621,7 +621,6 @@ template <typename R> class BatchRunner {
         DWF_REQUIRE(SB + nr * SS <= NSCALAR, DWF_EINVAL, "too many right-hand sides in one batch");
         mg.bscratch.ensure(nr);
         grow(mg.bcoef, sizeof(double2) * (size_t)nr * (MAX_RESTART + 2));
-        grow(mg.bscale, sizeof(double) * (size_t)nr);
     }
     static void grow(DevBuf &b, size_t bytes) {
         if (b.bytes < bytes) b.alloc(bytes);
@@ -1272,7 +1271,6 @@ template <typename R> class BatchRunner {
         auto any = [&]() { for (int r = 0; r < nr; ++r) if (act[r]) return true; return false; };
         std::vector<double2> Tm((size_t)nr * restart * restart), alpha((size_t)nr * restart);
         std::vector<double2> al(nr);
-        std::vector<double> scr(nr);
         long long active_iters = 0;
         int k = 0;
         while (k < restart && any()) {
@@ -1281,10 +1279,15 @@ template <typename R> class BatchRunner {
             for (int r = 0; r < nr; ++r)
                 for (int i = 0; i <= k; ++i) Tm[(size_t)r * restart * restart + i * restart + k] = make_double2(0, 0);
             // classical Gram-Schmidt of W_k against W_0 .. W_{k-1} (a second pass
-            // where the first removed 3/4 or more of |W_k|^2)
+            // where the first removed 3/4 or more of |W_k|^2), |W_k|^2 and
+            // <r, W_k> of the result behind it: one read by the host decides
+            // about the second pass and gives the step
+            constexpr int SN = 120;  // slots of |W_k|^2 (SN) and <r, W_k> (SN + 2, SN + 3)
+            T *pair[2] = {W[k], rr};
             for (int pass = 0; pass < 2; ++pass) {
                 multidot_b<T>(c, mg.bscratch, SB, SS, W.data(), k + 1, W[k], N, nr);
                 if (k > 0) multiaxpy_b<T>(c, W[k], W.data(), k, SB, SS, -1.0, N, nr);
+                multidot_b<T>(c, mg.bscratch, SB + SN, SS, pair, 2, W[k], N, nr);
                 read_block(sv);
                 bool again = false;
                 for (int r = 0; r < nr; ++r) {
@@ -1300,21 +1303,17 @@ template <typename R> class BatchRunner {
                 }
                 if (!again) break;
             }
-            // |W_k|^2 and <W_k, r> per right-hand side
-            norm2_b<T>(c, mg.bscratch, SB + 2, SS, W[k], N, nr);
-            T *wk = W[k];
-            multidot_b<T>(c, mg.bscratch, SB + 4, SS, &wk, 1, rr, N, nr);
-            read_block(sv);
+            GcrStep step;
             for (int r = 0; r < nr; ++r) {
                 const double *v = sv.data() + (size_t)r * SS;
-                const double ww = v[2];
+                const double ww = v[SN];
                 double2 &Td = Tm[(size_t)r * restart * restart + k * restart + k];
                 const bool ok = ww > 0.0 && std::isfinite(ww);
-                scr[r] = ok ? 1.0 / std::sqrt(ww) : 0.0;
+                step.scale[r] = ok ? 1.0 / std::sqrt(ww) : 0.0;
                 if (act[r] && ok) {
                     const double nw = std::sqrt(ww);
                     Td = make_double2(nw, 0.0);
-                    al[r] = make_double2(v[4] / nw, v[5] / nw);
+                    al[r] = make_double2(v[SN + 2] / nw, -v[SN + 3] / nw);  // <W_k, r> / |W_k|
                     const double r2 = rn[r] * rn[r] - (al[r].x * al[r].x + al[r].y * al[r].y);
                     rn[r] = r2 > 0 ? std::sqrt(r2) : 0.0;
                     ++active_iters;
@@ -1322,11 +1321,9 @@ template <typename R> class BatchRunner {
                     Td = make_double2(1.0, 0.0);
                     al[r] = make_double2(0.0, 0.0);
                 }
-                alpha[(size_t)r * restart + k] = al[r];
+                alpha[(size_t)r * restart + k] = step.al[r] = al[r];
             }
-            DWF_CUDA(cudaMemcpyAsync(mg.bcoef.p, al.data(), sizeof(double2) * nr, cudaMemcpyHostToDevice, c->stream));
-            DWF_CUDA(cudaMemcpyAsync(mg.bscale.p, scr.data(), sizeof(double) * nr, cudaMemcpyHostToDevice, c->stream));
-            gcr_wr_b<T>(c, W[k], rr, mg.bscale.as<double>(), mg.bcoef.as<double2>(), N, nr);
+            gcr_wr_b<T>(c, W[k], rr, step, N, nr);
             for (int r = 0; r < nr; ++r)
                 if (act[r] && rn[r] <= tol[r] * bn[r]) act[r] = 0;
             ++k;

@@ -63,7 +63,7 @@ struct MGState {
     BatchScratch bscratch;
     // the batched solve's coefficient arrays and the scratch of its coarsest
     // solves; kept between calls (every user runs on the context's stream)
-    DevBuf bcoef, bscale, cb_r, cb_Z, cb_W, cb_part;
+    DevBuf bcoef, cb_r, cb_Z, cb_W, cb_part;
     static constexpr int NSIDE = 3;
     DevBuf cs_r[NSIDE], cs_Z[NSIDE], cs_W[NSIDE], cs_part[NSIDE];
     mg_stats stats;
@@ -195,7 +195,12 @@ void normalised_b(dwf_ctx *c, double2 *out, const T *x, int base, int stride, in
 // a CG direction moved to a replaced residual: p = zt + c (p - z), c = |zt|^2 / |z|^2
 // from the slots izt, iz (with p = z + b p_old: zt + (|zt|^2 / |z_old|^2) p_old)
 template <typename T> void cg_redirect(dwf_ctx *c, T *p, const T *zt, const T *z, int izt, int iz, int64_t n);
-template <typename T> void gcr_wr_b(dwf_ctx *c, T *w, T *res, const double *sc, const double2 *al, int64_t n, int nrhs);
+// w_r *= scale[r];  res_r -= al[r] w_r (passed by value: no copy to the device)
+struct GcrStep {
+    double scale[32];
+    double2 al[32];
+};
+template <typename T> void gcr_wr_b(dwf_ctx *c, T *w, T *res, const GcrStep &step, int64_t n, int nrhs);
 template <typename T> void combo_b(dwf_ctx *c, T *x, T *const *V, int k, const double2 *g, int64_t n, int nrhs);
 
 // ---- blas2.cu ----  (host scalars; FP64 accumulate inside reductions)
