@@ -394,8 +394,8 @@ template <typename R> class Runner {
         Level &L = mg.lev[l];
         const mg_params &p = mg.p;
         const int64_t N = n(l);
-        L.vec64.alloc(sizeof(double2) * N * L.nadapt);
-        Qbuf<R>(L).alloc(sizeof(T) * N * L.nv);
+        if (L.vec64.bytes != sizeof(double2) * N * L.nadapt) L.vec64.alloc(sizeof(double2) * N * L.nadapt);
+        if (Qbuf<R>(L).bytes != sizeof(T) * N * L.nv) Qbuf<R>(L).alloc(sizeof(T) * N * L.nv);
         double2 *v = L.vec64.as<double2>();
         if (l == 0 && start) {
             DevBuf canon;
@@ -1616,9 +1616,43 @@ void mg_free(dwf_ctx *c) {
     c->mg = nullptr;
 }
 
+// Buffers of an earlier setup on the same lattice that the coming one would
+// allocate in exactly this size: the fine basis, the adaptive vectors and the
+// workspaces of the FP32 relaxation (allocating and freeing them took 10 ms of
+// 33 at 12^3 x 16 x 16, Nvec 24).  Nothing is kept that it does not need.
+static void keep_buffers(MGState &mg, MGState &old) {
+    Level &L = mg.lev[0], &O = old.lev[0];
+    const bool f32 = mg.p.smoother_prec == DWF_F32;
+    const size_t N = (size_t)L.lg.nelem;
+    auto take = [](DevBuf &to, DevBuf &from, size_t bytes) {
+        if (from.bytes == bytes) to = std::move(from);
+    };
+    take(L.vec64, O.vec64, sizeof(double2) * N * L.nadapt);
+    if (f32) take(L.Q32, O.Q32, sizeof(float2) * N * L.nv);
+    else take(L.Q64, O.Q64, sizeof(double2) * N * L.nv);
+    if (!f32 || !batch_on() || L.nadapt < 2 || L.nadapt > 32 || mg.p.setup_iters0 < 1) return;
+    // the workspaces of relax and of cgnr_b's form at this fifth extent
+    std::vector<int> used = {0, 2, 3, 8, 9, 10};
+    if (relax_zform(L.lg.g.Ls)) {
+        used.push_back(13);
+        for (int j = 0; j <= 8; ++j) used.push_back(100 + j);
+    } else {
+        used.insert(used.end(), {1, 5});
+    }
+    mg.wsb[0].resize(109);
+    for (int i : used)
+        if (i < (int)old.wsb[0].size()) take(mg.wsb[0][i], old.wsb[0][i], sizeof(float2) * N * L.nadapt);
+}
+
 dwf_status mg_setup_impl(dwf_ctx *c, int levels, const int *nvec, const int (*block)[4], const mg_params &p,
                          const void *start, bool start_on_host) {
-    mg_free(c);
+    // the previous setup's state, freed before anything new is allocated, but
+    // for the buffers this setup needs in the same size
+    struct Old {
+        MGState *p;
+        ~Old() { delete p; }
+    } old{c->mg};
+    c->mg = nullptr;
     DWF_REQUIRE(p.smoother_prec == DWF_F64 || p.smoother_prec == DWF_F32, DWF_EINVAL, "smoother_prec must be F64 or F32");
     DWF_REQUIRE(p.nu_post >= 0 && p.nu_pre >= 0 && p.coarse_restart >= 1 &&
                     p.outer_restart >= 1 && p.outer_restart <= MAX_RESTART && p.setup_sweep_iters >= 1 &&
@@ -1681,6 +1715,11 @@ dwf_status mg_setup_impl(dwf_ctx *c, int levels, const int *nvec, const int (*bl
             delete mg;
             throw;
         }
+    }
+    if (old.p) {
+        keep_buffers(*mg, *old.p);
+        delete old.p;
+        old.p = nullptr;
     }
     c->mg = mg;
     try {
