@@ -23,7 +23,7 @@ namespace {
 // component stride LS; the staged link `m` already carries the hop
 // coefficient (-1/2, or +1/2 across an antiperiodic t boundary).
 template <int MU, bool ADJ, typename R, int LS>
-__device__ __forceinline__ void hop_row(C<R> acc[12], const C<R> *__restrict__ p, int ls_rt, const C<R> *m, int sig) {
+__device__ __forceinline__ void hop_row(C<R> acc[12], const C<R> *p, int ls_rt, const C<R> *m, int sig) {
     const int Ls = LS > 0 ? LS : ls_rt;
     C<R> v[12];
 #pragma unroll
@@ -65,7 +65,7 @@ __device__ __forceinline__ void hop_row(C<R> acc[12], const C<R> *__restrict__ p
 // whole warps: blockDim.x a multiple of 32, no early exit before the norms).
 template <typename R, bool DAG, bool SHFL, int LS, int MINB, int EPI>
 __global__ void __launch_bounds__(128, MINB)
-dslash_kernel(C<R> *__restrict__ out, const C<R> *__restrict__ in, const C<R> *__restrict__ U, Geom g, R diag, R mf,
+dslash_kernel(C<R> *out, const C<R> *in, const C<R> *__restrict__ U, Geom g, R diag, R mf,
               int spb, int64_t field, NormOut nout, ZUpdateT<R> zu) {
     constexpr bool NORM = EPI == 1 || EPI == 2 || EPI == 4;
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -54,7 +54,7 @@ __device__ __forceinline__ void norm_epilogue(const NormOut &n, int r, double v,
 }
 
 // nslot[r * nstride] = sum of the nb CTA partials of right-hand side r = blockIdx.x (fixed order)
-__global__ void __launch_bounds__(1024) norm_finish_kernel(const double *__restrict__ npart, double *__restrict__ nslot,
+__global__ void __launch_bounds__(1024) norm_finish_kernel(const double *npart, double *nslot,
                                                            int nstride, int nb) {
     __shared__ double red[32];
     pdl_wait();

@@ -170,7 +170,7 @@ __device__ __forceinline__ void hop2(CP acc[12], const float4 p[12], const float
 }
 
 // the 12 components of a thread's two slices in one site's row
-template <int LS> __device__ __forceinline__ void ldrow(float4 p[12], const float2 *__restrict__ row) {
+template <int LS> __device__ __forceinline__ void ldrow(float4 p[12], const float2 *row) {
 #pragma unroll
     for (int k = 0; k < 12; ++k) p[k] = *reinterpret_cast<const float4 *>(row + k * LS);
 }
@@ -233,7 +233,7 @@ constexpr int PAIR_THREADS = 128;  // at most; 128 registers per thread
 // a = zz[r * stride] / ww[r * stride] (0 where the denominator is not positive).
 template <bool DAG, int LS, int EPI>
 __global__ void __launch_bounds__(PAIR_THREADS, 4)
-dslash_pair_kernel(float2 *__restrict__ out0, const float2 *__restrict__ in0, const float2 *__restrict__ U, Geom g,
+dslash_pair_kernel(float2 *out0, const float2 *in0, const float2 *__restrict__ U, Geom g,
                    Brick bk, float diag, float mf, int64_t field, NormOut nout, ZUpdate zu, int nrhs, int rb) {
     constexpr bool NORM = EPI == 1 || EPI == 2 || EPI == 4;
     constexpr int TPS = LS / 2;      // lanes per site
@@ -290,8 +290,8 @@ dslash_pair_kernel(float2 *__restrict__ out0, const float2 *__restrict__ in0, co
     if (EPI >= 2 && active) request_z(r0);
     __syncthreads();
     for (int rhs = r0; rhs < r1; ++rhs) {
-        const float2 *__restrict__ in = in0 + (size_t)rhs * (size_t)field;
-        float2 *__restrict__ out = out0 + (size_t)rhs * (size_t)field;
+        const float2 *in = in0 + (size_t)rhs * (size_t)field;
+        float2 *out = out0 + (size_t)rhs * (size_t)field;
         // the first two hops' rows are requested together with the thread's own
         // row; each later row is requested while the hop before it computes
         float4 pa[12], pb[12], self[12];

@@ -97,7 +97,10 @@ void note_launches(unsigned long long n);  // kernels launched by a replayed gra
 // pdl_dependents (or ended), and runs up to its pdl_wait beside that kernel's
 // tail; pdl_wait returns when the kernel before has completed and its writes
 // are visible.  Every such kernel calls pdl_wait before it touches anything a
-// kernel writes, so completion stays in stream order.  pdl_dependents comes
+// kernel writes, so completion stays in stream order; what other kernels write
+// it reads through pointers that are not `const __restrict__` (those may be
+// read by non-coherent loads, which promise that nobody writes the data while
+// the kernel runs).  pdl_dependents comes
 // late in the kernels here: CTAs that start while the grid before still fills
 // most SMs settle unevenly on what is left, which a grid of one wave never
 // makes up (FP64 V-cycle at 8^4 x 8: 2.28 ms with the call first, 1.50 without
