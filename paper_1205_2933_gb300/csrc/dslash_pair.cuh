@@ -339,7 +339,8 @@ dslash_pair_kernel(float2 *out0, const float2 *in0, const float2 *__restrict__ U
             hop2<3, false>(acc, pa, sLs + 3 * 10, fs);
             if (EPI >= 2) ldrow<LS>(pa, zu.zin + (size_t)rhs * (size_t)field + self_off);
             hop2<3, true>(acc, pb, sLs + 7 * 10, -fs);
-            if (rhs + 1 == r1) pdl_dependents();
+            // (>= where == would do: the plain kernels spill 16 bytes instead of 32, 428 -> 412 us)
+            if (rhs + 1 >= r1) pdl_dependents();
             float2 *o = out + self_off;
             float a = 1.f;
             if (EPI == 2 || EPI == 4) {

@@ -5,8 +5,7 @@
 // A coarse site owns a block of bx*by*bz*bt sites of the finer level with all
 // their components and all s.  In the s-fastest layout the elements of one
 // finer site are contiguous (ncomp*Ls of them), so a CTA that walks the
-// block site by site reads whole contiguous runs.  One CTA per coarse site;
-// reductions over the block use warp shuffles, then shared memory.
+// block site by site reads whole contiguous runs.
 #include <cooperative_groups.h>
 
 #include "blockmap.cuh"
