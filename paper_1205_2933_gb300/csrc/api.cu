@@ -106,6 +106,7 @@ dwf_status create_one(dwf_ctx **out, const int dims[4], int Ls, double M5, doubl
         DWF_CUDA(cudaGetDevice(&c->device));
         DWF_CUDA(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device));
         DWF_CUDA(cudaDeviceGetAttribute(&c->smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
+        DWF_CUDA(cudaDeviceGetAttribute(&c->l2_bytes, cudaDevAttrL2CacheSize, c->device));
         for (int i = 0; i < 4; ++i) c->g.L[i] = dims[i];
         c->g.Ls = Ls;
         c->g.V = (int64_t)dims[0] * dims[1] * dims[2] * dims[3];

@@ -175,6 +175,26 @@ template <int LS> __device__ __forceinline__ void ldrow(float4 p[12], const floa
     for (int k = 0; k < 12; ++k) p[k] = *reinterpret_cast<const float4 *>(row + k * LS);
 }
 
+// L2 priority of data that nobody reads again soon (first) or of any other
+__device__ __forceinline__ uint64_t l2_policy(int first) {
+    uint64_t f, n;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(f));
+    asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(n));
+    return first ? f : n;
+}
+
+__device__ __forceinline__ float4 ld_hint(const float4 *p, uint64_t policy) {
+    float4 v;
+    asm volatile("ld.global.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p), "l"(policy));
+    return v;
+}
+
+__device__ __forceinline__ void st_hint(float4 *p, const float4 &v, uint64_t policy) {
+    asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z),
+                 "f"(v.w), "l"(policy) : "memory");
+}
+
 // A warp holds 32 / (LS/2) whole sites (LS/2 lanes each, the lanes left over
 // idle), so that the fifth-dimension neighbours are lanes of the same warp.
 // A staged link takes 10 float2 (9 used) and a site LSTRIDE: the sites of one
@@ -337,7 +357,11 @@ dslash_pair_kernel(float2 *out0, const float2 *in0, const float2 *__restrict__ U
             hop2<2, false>(acc, pa, sLs + 2 * 10, fs);  ldrow<LS>(pa, in + nb(3, true));
             hop2<2, true>(acc, pb, sLs + 6 * 10, -fs);  ldrow<LS>(pb, in + nb(3, false));
             hop2<3, false>(acc, pa, sLs + 3 * 10, fs);
-            if (EPI >= 2) ldrow<LS>(pa, zu.zin + (size_t)rhs * (size_t)field + self_off);
+            if (EPI >= 2) {
+                const float2 *zp = zu.zin + (size_t)rhs * (size_t)field + self_off;
+#pragma unroll
+                for (int k = 0; k < 12; ++k) pa[k] = ld_hint(reinterpret_cast<const float4 *>(zp + k * LS), l2_policy(zu.stream));
+            }
             hop2<3, true>(acc, pb, sLs + 7 * 10, -fs);
             // (>= where == would do: the plain kernels spill 16 bytes instead of 32, 428 -> 412 us)
             if (rhs + 1 >= r1) pdl_dependents();
@@ -357,7 +381,9 @@ dslash_pair_kernel(float2 *out0, const float2 *in0, const float2 *__restrict__ U
                     re = make_float2(fmaf(a, pa[k].x, re.x), fmaf(a, pa[k].z, re.y));
                     im = make_float2(fmaf(a, pa[k].y, im.x), fmaf(a, pa[k].w, im.y));
                 }
-                *reinterpret_cast<float4 *>(o + k * LS) = make_float4(re.x, im.x, re.y, im.y);
+                const float4 v = make_float4(re.x, im.x, re.y, im.y);
+                if (EPI >= 2) st_hint(reinterpret_cast<float4 *>(o + k * LS), v, l2_policy(zu.stream));
+                else *reinterpret_cast<float4 *>(o + k * LS) = v;
                 if (NORM) nrm += re.x * re.x + im.x * im.x + re.y * re.y + im.y * im.y;
             }
             if (EPI >= 2 && rhs + 1 < r1) request_z(rhs + 1);
@@ -399,7 +425,12 @@ void dslash_pair_ls(dwf_ctx *c, float2 *out, const float2 *in, bool dag, int nrh
     const float diag = (float)(5.0 - c->M5), mf = (float)c->mf;
     const float2 *U = c->U32.as<float2>();
     const NormOut nout = nslot ? norm_out(c, grid, nrhs, nslot, nstride) : NormOut{};
-    const ZUpdate z = zu ? *zu : ZUpdate{nullptr, nullptr, nullptr, 0, 0};
+    ZUpdate z = zu ? *zu : ZUpdate{nullptr, nullptr, nullptr, 0, 0, 0};
+    // Fields that do not fit in L2 together: the second field and the output, each
+    // touched once, leave it first, so that the rows shared by neighbouring CTAs
+    // stay (V-cycle at 16^3 x 32 x 16, four sources: 22.5 -> 21.6 ms).  Fields that
+    // fit are read again by the next kernel: there it costs 1 % (8^3 x 16 x 16).
+    z.stream = 3 * (int64_t)nrhs * field * (int64_t)sizeof(float2) > c->l2_bytes;
 #define PL(D, E)                                                                                                  \
     launch_after(dslash_pair_kernel<D, LS, E>, grid, dim3(threads), smem, c->stream, out, in, U, g, bk, diag, mf, \
                  field, nout, z, nrhs, rb)

@@ -219,6 +219,7 @@ template <typename R> struct ZUpdateT {
     const double *ww;   // denominator of a at ww[r * stride]
     int stride;
     int add;            // 1: out = D in + a zin (EPI 4); 0: out = zin - a D^+ in (EPI 2)
+    int stream;         // paired kernel: zin and out leave L2 first
 };
 using ZUpdate = ZUpdateT<float>;
 
@@ -270,6 +271,7 @@ struct dwf_ctx {
     cudaStream_t stream = nullptr;
     int device = 0;
     int sm_count = 0;
+    int l2_bytes = 0;
     int smem_optin = 0;  // shared memory a CTA may opt in to
     dwf_status sticky = DWF_OK;
     dwf::Brick brick[2];  // of the paired Dslash with 64 and 128 threads per CTA
