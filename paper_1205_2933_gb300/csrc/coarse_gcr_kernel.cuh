@@ -557,7 +557,9 @@ template <typename R, typename LT, int NV, int NPTS> void launch_nv(dwf_ctx *c, 
     const SmemPlan<R, LT, NV, NPTS> plan(a.g.V, a.restart, max_ctas, (size_t)c->smem_optin - 4096);
     if (plan.total <= (size_t)c->smem_optin - 4096) {
         void *fn = (void *)coarse_gcr_smem_kernel<R, LT, NV, NPTS>;
-        DWF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.total));
+        // one value whatever this launch needs: the lattices of a batch launch
+        // from several threads, and the limit belongs to the kernel
+        DWF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, c->smem_optin - 4096));
         int spc = (int)plan.spc, cached = plan.cached ? 1 : 0;
         void *kargs[] = {&a, &spc, &cached};
         DWF_CUDA(coop_launch(c, fn, dim3((unsigned)((a.g.V + spc - 1) / spc)), dim3(CT), kargs, plan.total));

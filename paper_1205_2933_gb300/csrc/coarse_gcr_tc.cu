@@ -740,7 +740,12 @@ void launch_tc(dwf_ctx *c, const Level &L, float2 *x, const float2 *b, int nb, f
     void *kargs[] = {&a};
     void *fn = tc_kernel_fn<NV>();
     const size_t smem = tc_smem<NV>(nb);
-    DWF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // one value whatever this launch needs: the lattices of a batch launch from
+    // several threads, and the limit belongs to the kernel
+    cudaFuncAttributes fa;
+    DWF_CUDA(cudaFuncGetAttributes(&fa, fn));
+    DWF_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  c->smem_optin - (int)fa.sharedSizeBytes));
     int per_sm = 0;
     DWF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, TCT, smem));
     DWF_REQUIRE(per_sm >= 1, DWF_ECUDA, "tensor-core coarse solver cannot be co-resident");

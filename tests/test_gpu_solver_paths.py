@@ -159,3 +159,18 @@ def test_setup_after_setup(G, prec, tol):
             assert ((a - b).norm() / b.norm()).item() < tol
         new.close()
     old.close()
+
+
+def test_coarse_shapes_of_a_batch_share_a_kernel(G):
+    """Lattices of one context solve from threads of their own, with the same
+    coarsest kernel at different shared-memory needs: one's launch must not
+    lower what another's may ask for."""
+    dims = [(8, 8, 8, 8), (4, 4, 4, 4), (4, 4, 4, 8)]
+    bc = G.BatchContext(dims, 4, 1.8, 0.1, [torch.from_numpy(I.epsilon_links(d, 0.3, 1)).cuda() for d in dims])
+    p = M._params(G, setup_iters0=16, smoother_prec=1, coarse_prec=[1])
+    G.mg_setup(bc.h, 2, [8], [(2, 2, 2, 2)], p)
+    b = torch.from_numpy(np.concatenate([I.gaussian_source(d, 4, 5).reshape(-1) for d in dims])).cuda()
+    for _ in range(10):
+        x = torch.zeros_like(b)
+        assert G.mg_solve(bc.h, b, x, 1e-8).true_res <= 1e-8
+    bc.close()
