@@ -52,8 +52,8 @@ FINE_BYTES_F32 = 204   # algorithmic bytes per 5D site of the FP32 Dslash
 # output norms (the instantiation of nearly all timed launches) per 2,097,152
 # 5D sites (one 16^3x32x16 field), from an ncu capture of a two-field launch on
 # 16^3x16x16; None until the kernel as it stands has been captured
-DSLASH_TRAFFIC_PER_FIELD = 425732864  # 251.68 MB read + 174.05 MB written
-DSLASH_Z_TRAFFIC_PER_FIELD = 630616832  # 453.86 MB read + 176.76 MB written
+DSLASH_TRAFFIC_PER_FIELD = 452406272  # 256.74 MB read + 195.67 MB written
+DSLASH_Z_TRAFFIC_PER_FIELD = 668735488  # 471.54 MB read + 197.20 MB written
 FINE_BYTES_F64 = 408
 FINE_BYTES_F32_Z = FINE_BYTES_F32 + 96  # the fused residual kernels also read b (or z) at every 5D site
 # fine-operator applications per solve of this workload on the GPU path (FP32 and

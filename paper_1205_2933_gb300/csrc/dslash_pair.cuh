@@ -200,8 +200,9 @@ __device__ __forceinline__ void st_hint(float4 *p, const float4 &v, uint64_t pol
 // A staged link takes 10 float2 (9 used) and a site LSTRIDE: the sites of one
 // warp start 4 banks apart and their reads of the same elements do not collide.
 //
-// What bounds the kernel is the L1 data path, 76 % of its wavefronts busy at
-// 450 us for four fields of 16^3 x 32 x 16 (DRAM at 54 % of the copy rate): nine
+// What bounds the kernel is the L1 data path, 76 % of its wavefronts busy when
+// four fields of 16^3 x 32 x 16 took 450 us, 69 % at the 412 us they take now
+// (DRAM at 242 / 412 = 59 % of the copy rate): nine
 // rows of 96 bytes per 5D site are read, and the rows in flight (16 warps x 2)
 // exceed L1, so 87 % of them are also filled whatever the shape of the CTA's
 // sites.  Hence: the links as 16-byte loads of two elements instead of one

@@ -1151,7 +1151,7 @@ template <typename R> class BatchRunner {
     // epilogues, x and the next direction formed once per chunk, the residual
     // computed explicitly where it is tested.  Two Dslash launches and their
     // norm sums per iteration instead of eight launches: at 8^3 x 16 x 16
-    // 48 us per iteration against 92 us.  A reliable update moves the direction to
+    // 46 us per iteration against 92 us.  A reliable update moves the direction to
     // the new residual's z and computes its w afresh.
     static constexpr int CG_FIELDS = CHUNK + 7;  // FP32 fields it works on
     dwf_status cg_solve(const double2 *b, double2 *x, double tol, int maxiter, int cycle, mg_stats &st) {
@@ -1475,9 +1475,10 @@ bool batch_on() {
 
 // The batched path covers V-cycles on two levels with nu_1 = 0, one right-hand
 // side included (its smoother then needs 2 launches per step instead of 6: a
-// FP32 V-cycle at 8^3 x 16 x 16 in 1.07 ms instead of 1.50; an FP64 one at
-// 8^4 x 8 in 1.43 ms instead of 1.65), FP64 always one at a time.  An FP16 basis copy is used only by
-// the other V-cycle.  DWF_BATCH=0 in the environment turns it off.
+// FP32 V-cycle at 8^3 x 16 x 16 in 1.07 ms instead of 1.50 when it moved here,
+// 0.77 now; an FP64 one at 8^4 x 8 in 1.43 ms instead of 1.65), FP64 always
+// one at a time.  An FP16 basis copy is used only by the other V-cycle.
+// DWF_BATCH=0 in the environment turns it off.
 template <typename R> bool batch_eligible(const MGState &mg, int nrhs) {
     return (nrhs > 1 || !mg.lev[0].Q16.p) && batch_on() && mg.nlevels == 2 && mg.p.nu_pre == 0 &&
            mg.p.outer_restart <= 32 && mg.p.coarsen == 0;
