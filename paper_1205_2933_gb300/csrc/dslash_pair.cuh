@@ -418,7 +418,11 @@ void dslash_pair_ls(dwf_ctx *c, float2 *out, const float2 *in, bool dag, int nrh
         const double w = (double)bk.count * ((nrhs + n - 1) / n) / slots;
         return (w < 4.0 ? std::ceil(w) : w) * (0.25 + n);
     };
-    const int rb = nrhs > 1 && cost(2) <= cost(1) ? 2 : 1;
+    int rb = nrhs > 1 && cost(2) <= cost(1) ? 2 : 1;
+    // at the short fifth extents the links are a larger share of the work: four
+    // where that still leaves three waves of CTAs (16^3 x 32 x 8, three fields:
+    // 248 -> 216 us; x 4, twelve fields: 799 -> 761; at Ls 32 four lose 3 %)
+    if (LS <= 8 && nrhs > 2 && (double)bk.count * ((nrhs + 3) / 4) / slots >= 3.0) rb = 4;
     DWF_REQUIRE(bk.count < ((int64_t)1 << 31), DWF_EINVAL, "paired Dslash: grid too large");
     dim3 grid((unsigned)bk.count, (unsigned)((nrhs + rb - 1) / rb));
     const size_t smem = (size_t)spb * LSTRIDE * sizeof(float2);

@@ -174,3 +174,17 @@ def test_coarse_shapes_of_a_batch_share_a_kernel(G):
         x = torch.zeros_like(b)
         assert G.mg_solve(bc.h, b, x, 1e-8).true_res <= 1e-8
     bc.close()
+
+
+@pytest.mark.parametrize("Ls,nrhs", [(8, 3), (4, 5)])
+def test_apply_of_several_fields_per_link(G, Ls, nrhs):
+    """Large grids at short fifth extents: each field as when it is alone, bit for bit."""
+    ctx = _ctx((16, 16, 16, 32), Ls)
+    n = ctx.field_elems
+    f = torch.randn(nrhs * n, dtype=torch.complex64, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    out, one = torch.empty_like(f), torch.empty(n, dtype=f.dtype, device="cuda")
+    G.dwf_apply(ctx.h, out, f, G.DWF_F32, False, nrhs)
+    for r in range(nrhs):
+        G.dwf_apply(ctx.h, one, f[r * n:(r + 1) * n].clone(), G.DWF_F32, False, 1)
+        assert torch.equal(out[r * n:(r + 1) * n], one)
+    ctx.close()
