@@ -1063,7 +1063,9 @@ template <typename R> class BatchRunner {
     }
 
     void vcycle_b(T *x, const T *b) {
-        if (!mg.p.graph || c->gate) return vcycle_body(x, b);
+        // (a coarsest solve that is not one of the fused kernels reads its scalars on
+        // the host, which a capture does not allow)
+        if (!mg.p.graph || c->gate || !coarse_gcr_fused_ok(mg.lev[1], mg.p.coarse_restart)) return vcycle_body(x, b);
         for (auto &g : graphs)
             if (g.x == x && g.b == b && g.nr == nr) return replay(g);
         if (std::find(eager_nr.begin(), eager_nr.end(), nr) == eager_nr.end()) {

@@ -1,0 +1,41 @@
+"""Calls at the ends of what the library accepts: parameters above the limit of
+a fused kernel, and what the statistics say of such calls."""
+import numpy as np
+import pytest
+
+import paper_1205_2933_gb300.inputs as I
+import test_gpu_mg as M
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def G():
+    from paper_1205_2933_gb300 import dwfmg
+    return dwfmg
+
+
+def _setup(G, dims=(4, 4, 4, 4), Ls=8, nvec=8, block=(2, 2, 2, 2), **kw):
+    from gpu_util import ctx_for
+    ctx = ctx_for(I.epsilon_links(dims, 0.3, 1), dims, Ls, 1.8, 0.1)
+    p = M._params(G, **kw)
+    start = torch.from_numpy(I.random_vectors(nvec // 2, dims, Ls, 3)).cuda()
+    G.mg_setup(ctx.h, 2, [nvec], [block], p, start)
+    return ctx
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["f64", "f32"])
+@pytest.mark.parametrize("nrhs", [1, 3])
+def test_coarse_restart_beyond_the_fused_solver(G, prec, nrhs):
+    """coarse_restart up to 64 is accepted; above 32 the coarsest solve runs
+    launch by launch with host reads, which no graph may hold.  A solve of
+    several V-cycles with the default parameters reaches its tolerance."""
+    dims, Ls = (4, 4, 4, 4), 8
+    ctx = _setup(G, dims, Ls, setup_iters0=8, setup_sweeps=0, smoother_prec=prec, coarse_prec=[prec], coarse_restart=40)
+    b = np.concatenate([I.gaussian_source(dims, Ls, 5 + r).reshape(-1) for r in range(nrhs)])
+    b = torch.from_numpy(b).cuda()
+    x = torch.zeros_like(b)
+    st = G.mg_solve(ctx.h, b, x, 1e-8, nrhs)
+    assert st.true_res <= 1e-8 and st.iters > 2 * nrhs
+    ctx.close()
