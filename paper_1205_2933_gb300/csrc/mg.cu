@@ -1564,7 +1564,7 @@ dwf_status solve_t(dwf_ctx *c, MGState &mg, double2 *b, double2 *x, double tol, 
             BatchRunner<R> br(c, mg, nb);
             dwf_status s = br.solve(b + (size_t)r0 * N, x + (size_t)r0 * N, tol, st);
             if (s != DWF_OK && worst == DWF_OK) worst = s;
-            c0 += br.one.fused_iters(1);
+            c0 += br.one.fused_iters(1) + br.one.coarse_applies[1];
         }
         st.coarse_applies[1] += c0;
         return worst;

@@ -39,3 +39,19 @@ def test_coarse_restart_beyond_the_fused_solver(G, prec, nrhs):
     st = G.mg_solve(ctx.h, b, x, 1e-8, nrhs)
     assert st.true_res <= 1e-8 and st.iters > 2 * nrhs
     ctx.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["f64", "f32"])
+@pytest.mark.parametrize("nrhs", [1, 3])
+@pytest.mark.parametrize("restart", [16, 40])
+def test_coarse_applications_are_counted(G, prec, nrhs, restart):
+    """Each outer iteration runs at least one coarsest iteration, by the fused
+    solver or launch by launch: the statistics count them in both."""
+    dims, Ls = (4, 4, 4, 4), 8
+    ctx = _setup(G, dims, Ls, setup_iters0=8, setup_sweeps=0, smoother_prec=prec, coarse_prec=[prec],
+                 coarse_restart=restart, graph=0, outer_maxiter=4, outer_restart=4)
+    b = np.concatenate([I.gaussian_source(dims, Ls, 5 + r).reshape(-1) for r in range(nrhs)])
+    b = torch.from_numpy(b).cuda()
+    st = G.mg_solve(ctx.h, b, torch.zeros_like(b), 1e-14, nrhs, check=False)
+    assert st.iters == 4 * nrhs and st.coarse_applies[1] >= st.iters
+    ctx.close()
