@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(CT) coarse_gcr_kernel(Args<R, LT> a) {
 
 // ---- the solver with its vectors in shared memory ---------------------------
 //
-// Sums that cross threads and CTAs: FP64 for FP64 fields; for FP32 fields the
+// Sums that cross threads and CTAs: FP64 for FP64 fields (and |b|^2); for FP32 fields the
 // unevaluated sum of two FP32 numbers (about 48 bits), because an FP64 addition
 // takes this chip's SM as long as 64 FP32 ones and every CTA adds up all
 // partials of a reduction.
@@ -385,7 +385,6 @@ __global__ void __launch_bounds__(CT) coarse_gcr_smem_kernel(Args<R, LT> a, int 
     C<R> *sin = reinterpret_cast<C<R> *>(sm + vec * (2 * a.restart + 2));
     C<R> *sp = reinterpret_cast<C<R> *>(sm + vec * (2 * a.restart + 2) + stage);
     unsigned char *sl = sm + vec * (2 * a.restart + 2) + 2 * stage;
-    AccC<A> *part = reinterpret_cast<AccC<A> *>(a.part);
     C<R> *pub = a.r;  // the published vector
 
     if (cached) {
@@ -419,11 +418,13 @@ __global__ void __launch_bounds__(CT) coarse_gcr_smem_kernel(Args<R, LT> a, int 
     };
     // tot[i] = the sum over all CTAs of <u_i, v_i>, i < n, u_i and v_i given by
     // the index; the partials in region `reg`, which no CTA reads any more
-    auto reduce = [&](int n, int reg, auto u, auto v) {
-        AccC<A> *pr = part + (size_t)reg * (MAXR + 2) * nb;
+    // (sums of the type of `zero`)
+    auto reduce = [&](auto zero, int n, int reg, auto u, auto v) {
+        using S = decltype(zero);
+        AccC<S> *pr = reinterpret_cast<AccC<S> *>(a.part) + (size_t)reg * (MAXR + 2) * nb;
         for (int i = warp; i < n; i += CT / 32) {
             const C<R> *ui = u(i), *vi = v(i);
-            AccC<A> s;
+            AccC<S> s;
             acc_init(s.re);
             acc_init(s.im);
             for (int e = lane; e < own; e += 32) {
@@ -443,12 +444,12 @@ __global__ void __launch_bounds__(CT) coarse_gcr_smem_kernel(Args<R, LT> a, int 
         __threadfence();
         grid.sync();
         for (int i = warp; i < n; i += CT / 32) {
-            AccC<A> s;
+            AccC<S> s;
             acc_init(s.re);
             acc_init(s.im);
             for (int k = lane; k < nb; k += 32) {
                 const float4 w = __ldcg(reinterpret_cast<const float4 *>(pr + (size_t)i * nb + k));
-                const AccC<A> t = *reinterpret_cast<const AccC<A> *>(&w);
+                const AccC<S> t = *reinterpret_cast<const AccC<S> *>(&w);
                 acc_add(s.re, t.re);
                 acc_add(s.im, t.im);
             }
@@ -469,8 +470,22 @@ __global__ void __launch_bounds__(CT) coarse_gcr_smem_kernel(Args<R, LT> a, int 
         pub[e0 + e] = v;
     }
     __syncthreads();
-    reduce(1, 0, [&](int) { return r; }, [&](int) { return r; });
-    const double bn2 = tot[0].x;
+    reduce(0.0, 1, 0, [&](int) { return r; }, [&](int) { return r; });
+    double bn2 = tot[0].x;
+    // FP32 fields: the solve runs on b scaled by the power of two that brings |b|
+    // near 1, so that the FP32 products above neither vanish nor overflow
+    // whatever b's size; x is scaled back at the end (both exact)
+    R up = 1, down = 1, up2 = 1, down2 = 1;  // each in two factors, which FP32 holds
+    if (sizeof(R) == 4 && bn2 > 0.0 && isfinite(bn2)) {
+        const int e = ((__double2hiint(bn2) >> 20) - 1023) >> 1, h = e >> 1;  // |b|^2 is no FP64 denormal
+        auto pow2 = [](int n) { return (R)__int_as_float((n + 127) << 23); };
+        up = pow2(-h);
+        up2 = pow2(h - e);
+        down = pow2(h);
+        down2 = pow2(e - h);
+        bn2 *= __hiloint2double((1023 - 2 * e) << 20, 0);
+        for (int i = tid; i < own; i += CT) pub[e0 + i] = r[i] = up2 * (up * r[i]);
+    }
     double rn2 = bn2;
     int it = 0, k = 0;
     if (bn2 > 0.0) {
@@ -486,7 +501,7 @@ __global__ void __launch_bounds__(CT) coarse_gcr_smem_kernel(Args<R, LT> a, int 
             auto V = [&](int i) { return i <= k ? w : r; };
             double ww = 0.0, wrx = 0.0, wry = 0.0;
             for (int pass = 0; pass < 2; ++pass) {
-                reduce(k + 2, pass, U, V);
+                reduce(A{}, k + 2, pass, U, V);
                 ww = tot[k].x;
                 wrx = tot[k + 1].x;
                 wry = tot[k + 1].y;
@@ -535,10 +550,10 @@ __global__ void __launch_bounds__(CT) coarse_gcr_smem_kernel(Args<R, LT> a, int 
                 apply(r);
                 for (int e = tid; e < own; e += CT) {
                     const C<R> v = a.b[e0 + e];
-                    r[e] = v - r[e];
+                    r[e] = up2 * (up * v) - r[e];
                 }
                 __syncthreads();
-                reduce(1, 0, [&](int) { return r; }, [&](int) { return r; });
+                reduce(A{}, 1, 0, [&](int) { return r; }, [&](int) { return r; });
                 for (int e = tid; e < own; e += CT) pub[e0 + e] = r[e];
                 rn2 = tot[0].x;
                 k = 0;
@@ -546,7 +561,7 @@ __global__ void __launch_bounds__(CT) coarse_gcr_smem_kernel(Args<R, LT> a, int 
             }
         }
     }
-    for (int e = tid; e < own; e += CT) a.x[e0 + e] = x[e];
+    for (int e = tid; e < own; e += CT) a.x[e0 + e] = down2 * (down * x[e]);
     if (blockIdx.x == 0 && tid == 0) atomicAdd(a.iters, it);
 }
 
