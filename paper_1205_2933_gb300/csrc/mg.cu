@@ -398,12 +398,19 @@ template <typename R> class Runner {
         if (Qbuf<R>(L).bytes != sizeof(T) * N * L.nv) Qbuf<R>(L).alloc(sizeof(T) * N * L.nv);
         double2 *v = L.vec64.as<double2>();
         if (l == 0 && start) {
+            // packed from where they are, unless a kernel cannot read them there:
+            // on the host, on another device, or off a 16-byte boundary
+            cudaPointerAttributes at{};
+            if (!start_on_host) DWF_CUDA(cudaPointerGetAttributes(&at, start));
+            const bool direct = !start_on_host && ((uintptr_t)start & 15) == 0 &&
+                                (at.type == cudaMemoryTypeManaged || at.device == c->device);
             DevBuf canon;
-            if (start_on_host) {
+            if (!direct) {
                 canon.alloc(sizeof(double2) * N * L.nadapt);
-                DWF_CUDA(cudaMemcpyAsync(canon.p, start, canon.bytes, cudaMemcpyHostToDevice, c->stream));
+                DWF_CUDA(cudaMemcpyAsync(canon.p, start, canon.bytes,
+                                         start_on_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, c->stream));
             }
-            pack(c, v, start_on_host ? canon.as<double2>() : (const double2 *)start, DWF_F64, L.nadapt);
+            pack(c, v, direct ? (const double2 *)start : canon.as<double2>(), DWF_F64, L.nadapt);
             DWF_CUDA(cudaStreamSynchronize(c->stream));
         } else {
             gauss_fill<double2>(c, v, L.nadapt, N, L.lg.g.Ls, L.lg.g.V, l == 0, p.seed + (uint32_t)l, 4u);

@@ -55,3 +55,28 @@ def test_coarse_applications_are_counted(G, prec, nrhs, restart):
     st = G.mg_solve(ctx.h, b, torch.zeros_like(b), 1e-14, nrhs, check=False)
     assert st.iters == 4 * nrhs and st.coarse_applies[1] >= st.iters
     ctx.close()
+
+
+@pytest.mark.parametrize("where", ["host", "device"])
+def test_start_vectors_off_a_16_byte_boundary(G, where):
+    """Start vectors may lie at any 8-byte boundary, on the device as on the host."""
+    from gpu_util import ctx_for
+    dims, Ls, nvec = (4, 4, 4, 4), 4, 8
+    start = I.random_vectors(nvec // 2, dims, Ls, 3).reshape(-1)
+    if where == "device":
+        buf = torch.empty(2 * start.size + 2, dtype=torch.float64, device="cuda")
+        off = buf[1:1 + 2 * start.size]
+        off.copy_(torch.from_numpy(start.view(np.float64)))
+    else:
+        buf = np.empty(2 * start.size + 2)
+        off = buf[1:1 + 2 * start.size]
+        off[:] = start.view(np.float64)
+    q = []
+    for s in (torch.from_numpy(start).cuda(), off):
+        ctx = ctx_for(I.epsilon_links(dims, 0.3, 1), dims, Ls, 1.8, 0.1)
+        G.mg_setup(ctx.h, 2, [nvec], [(2, 2, 2, 2)], M._params(G, setup_iters0=4, setup_sweeps=0), s)
+        q.append(torch.empty(nvec * ctx.field_elems, dtype=torch.complex128, device="cuda"))
+        G.mg_get_vectors(ctx.h, 0, q[-1])
+        torch.cuda.synchronize()
+        ctx.close()
+    assert torch.equal(q[0], q[1])
