@@ -581,7 +581,7 @@ template <typename R, typename LT, int NV, int NPTS> void launch_nv(dwf_ctx *c, 
         return;
     }
     void *kargs[] = {&a};
-    const int64_t nblk = std::max<int64_t>(1, std::min<int64_t>((a.g.V * NV + CT - 1) / CT, c->sm_count));
+    const int64_t nblk = std::max<int64_t>(1, std::min<int64_t>((a.g.V * NV + CT - 1) / CT, max_ctas));
     void *fn = (void *)coarse_gcr_kernel<R, LT, NV, NPTS>;
     int per_sm = 0;
     DWF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, CT, 0));

@@ -80,3 +80,37 @@ def test_start_vectors_off_a_16_byte_boundary(G, where):
         torch.cuda.synchronize()
         ctx.close()
     assert torch.equal(q[0], q[1])
+
+
+SIDE = """
+import numpy as np, torch
+import paper_1205_2933_gb300.inputs as I
+import test_gpu_mg as M
+from paper_1205_2933_gb300 import dwfmg as G
+from gpu_util import ctx_for
+dims, Ls, nvec, nr = (8, 6, 4, 6), 4, 24, 4
+ctx = ctx_for(I.epsilon_links(dims, 0.3, 1), dims, Ls, 1.8, 0.1)
+p = M._params(G, setup_iters0=0, setup_sweeps=0, smoother_prec=1, coarse_prec=[1], coarsest_tol=0.0, coarsest_maxiter=12)
+G.mg_setup(ctx.h, 2, [nvec], [(1, 1, 1, 1)], p, torch.from_numpy(I.random_vectors(nvec // 2, dims, Ls, 3)).cuda())
+b = torch.cat([torch.from_numpy(I.gaussian_source(dims, Ls, 40 + r).reshape(-1)).cuda() for r in range(nr)])
+x, y, n = torch.empty_like(b), torch.empty_like(b), ctx.field_elems
+G.mg_vcycle_batch(ctx.h, x, b, nr)
+for r in range(nr):
+    G.mg_vcycle(ctx.h, y[r * n:(r + 1) * n], b[r * n:(r + 1) * n])
+torch.cuda.synchronize()
+print("err", ((x - y).norm() / y.norm()).item())
+"""
+
+
+def test_coarsest_solves_side_by_side():
+    """Three coarsest solves at a time, each on a third of the SMs, where a
+    third of them cannot hold the vectors (1152 sites x 24, 34 vectors): as one
+    solve at a time to FP32 rounding (12 coarsest iterations, 8 smoothing steps)."""
+    import os
+    import subprocess
+    import sys
+    here = os.path.dirname(os.path.abspath(__file__))
+    env = dict(os.environ, DWF_COARSE_BATCH="0", PYTHONPATH=os.pathsep.join([os.path.dirname(here), here]))
+    out = subprocess.run([sys.executable, "-c", SIDE], env=env, capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stderr[-2000:]
+    assert float(out.stdout.split()[-1]) < 1e-4
