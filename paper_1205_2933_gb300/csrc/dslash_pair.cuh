@@ -327,24 +327,22 @@ dslash_pair_kernel(float2 *out0, const float2 *in0, const float2 *__restrict__ U
         const int lprev = base + (j == 0 ? TPS - 1 : j - 1);
         const float c_up1 = (s0 + 1 == LS - 1) ? mf : -1.f;  // s1 + 1 wraps to s = 0
         const float c_dn0 = (s0 == 0) ? mf : -1.f;           // s0 - 1 wraps to s = Ls-1
+        // (diag psi joins them in one fused operation: rounded on its own, the largest
+        // term of the sum would raise the kernel's error by 4 %)
         CP acc[12];
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            acc[k].re = pk(diag * self[k].x, diag * self[k].z);
-            acc[k].im = pk(diag * self[k].y, diag * self[k].w);
-        }
+        const P2 dg = pk(diag, diag);
 #pragma unroll
         for (int q = 0; q < 6; ++q) {
             // from s+1: slice s0 takes own s1 (coefficient -1), slice s1 takes s0 of the next lane
             const float4 su = self[up_lo + q];
             const float nx = __shfl_sync(0xffffffffu, su.x, lnext), ny = __shfl_sync(0xffffffffu, su.y, lnext);
-            acc[up_lo + q].re = add2(acc[up_lo + q].re, pk(-su.z, c_up1 * nx));
-            acc[up_lo + q].im = add2(acc[up_lo + q].im, pk(-su.w, c_up1 * ny));
+            acc[up_lo + q].re = fma2(dg, pk(su.x, su.z), pk(-su.z, c_up1 * nx));
+            acc[up_lo + q].im = fma2(dg, pk(su.y, su.w), pk(-su.w, c_up1 * ny));
             // from s-1: slice s0 takes s1 of the previous lane, slice s1 takes own s0 (coefficient -1)
             const float4 sd = self[dn_lo + q];
             const float pz = __shfl_sync(0xffffffffu, sd.z, lprev), pw = __shfl_sync(0xffffffffu, sd.w, lprev);
-            acc[dn_lo + q].re = add2(acc[dn_lo + q].re, pk(c_dn0 * pz, -sd.x));
-            acc[dn_lo + q].im = add2(acc[dn_lo + q].im, pk(c_dn0 * pw, -sd.y));
+            acc[dn_lo + q].re = fma2(dg, pk(sd.x, sd.z), pk(c_dn0 * pz, -sd.x));
+            acc[dn_lo + q].im = fma2(dg, pk(sd.y, sd.w), pk(c_dn0 * pw, -sd.y));
         }
         if (!NORM && !active) continue;
         float nrm = 0.f;
