@@ -110,20 +110,50 @@ __global__ void multiaxpy_b_kernel(T *__restrict__ w, MArgs<T> a, const double *
 //   r:  a = s[izz] / s[iww]; r -= a w
 //   px: a as above, b = s[inew] / s[izz]; x += a p; p = z + b p
 //   x:  x += a p (the last iteration, whose residual is not needed)
+//   p:  b as above; p' = z + b p
+// r and p stand between two Dslash kernels and launch as their dependents
+// (launch_after), hence the wait and the plain pointers: a FP32 V-cycle of one
+// field of 8^3 x 16 x 16, 15 of each, takes 0.99 ms, with ordinary launches and
+// 8-byte accesses 1.14.  Bound by three passes over the field (L2 or DRAM) and
+// the launch.
 template <typename T>
-__global__ void cg_r_b_kernel(T *rout, const T *rin, const T *__restrict__ w, const double *__restrict__ s, int base,
-                              int stride, int izz, int iww, int64_t n) {
+__global__ void cg_r_b_kernel(T *rout, const T *rin, const T *w, const double *s, int base, int stride, int izz, int iww,
+                              int64_t n) {
     using R = typename RealB<T>::type;
+    pdl_wait();
     const int r = blockIdx.y;
     const size_t off = (size_t)r * n;
     const double ww = s[base + r * stride + iww];
     const R a = ww > 0.0 ? (R)(s[base + r * stride + izz] / ww) : R(0);
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        T rv = rin[off + i];
-        const T wv = w[off + i];
-        rv.x -= a * wv.x;
-        rv.y -= a * wv.y;
-        rout[off + i] = rv;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n / Pack<T>::N; i += (int64_t)gridDim.x * blockDim.x) {
+        Pack<T> rv = ldp(rin + off, i);
+        const Pack<T> wv = ldp(w + off, i);
+#pragma unroll
+        for (int e = 0; e < Pack<T>::N; ++e) {
+            rv.e[e].x -= a * wv.e[e].x;
+            rv.e[e].y -= a * wv.e[e].y;
+        }
+        stp(rout + off, i, rv);
+    }
+}
+template <typename T>
+__global__ void cg_p_b_kernel(T *pout, const T *pin, const T *z, const double *s, int base, int stride, int izz, int inew,
+                              int64_t n) {
+    using R = typename RealB<T>::type;
+    pdl_wait();
+    const int r = blockIdx.y;
+    const size_t off = (size_t)r * n;
+    const double zz = s[base + r * stride + izz];
+    const R b = zz > 0.0 ? (R)(s[base + r * stride + inew] / zz) : R(0);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n / Pack<T>::N; i += (int64_t)gridDim.x * blockDim.x) {
+        Pack<T> pv = ldp(pin + off, i);
+        const Pack<T> zv = ldp(z + off, i);
+#pragma unroll
+        for (int e = 0; e < Pack<T>::N; ++e) {
+            pv.e[e].x = zv.e[e].x + b * pv.e[e].x;
+            pv.e[e].y = zv.e[e].y + b * pv.e[e].y;
+        }
+        stp(pout + off, i, pv);
     }
 }
 template <typename T>
@@ -274,9 +304,10 @@ __global__ void combo_b_kernel(T *__restrict__ x, MArgs<T> a, const double2 *__r
 // that basis: x = sum_k a_k p_k and p_k = z_k + b_{k-1} p_{k-1} give
 // g_{k-1} = a_{k-1}, g_j = a_j + b_j g_{j+1}, where a_j = |z_j|^2 / |w_j|^2
 // and b_j = |z_{j+1}|^2 / |z_j|^2 come from the scalar slots zb + j and wb + j.
+// directions: the Z_j are the p_j themselves, g_j = a_j.
 template <typename T>
 __global__ void cg_combine_b_kernel(T *__restrict__ x, MArgs<T> a, const double *__restrict__ s, int base, int stride,
-                                    int zb, int wb, int64_t n) {
+                                    int zb, int wb, int directions, int64_t n) {
     using R = typename RealB<T>::type;
     __shared__ R gam[32];
     __shared__ double al[32], be[32];
@@ -287,7 +318,7 @@ __global__ void cg_combine_b_kernel(T *__restrict__ x, MArgs<T> a, const double 
         const double *sr = s + base + (size_t)r * stride;
         const double zz = sr[zb + j], ww = sr[wb + j];
         al[j] = ww > 0.0 ? zz / ww : 0.0;
-        be[j] = (j + 1 < a.k && zz > 0.0) ? sr[zb + j + 1] / zz : 0.0;
+        be[j] = (!directions && j + 1 < a.k && zz > 0.0) ? sr[zb + j + 1] / zz : 0.0;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -488,7 +519,14 @@ void multiaxpy_b(dwf_ctx *c, T *w, T *const *V, int k, int base, int stride, dou
 template <typename T>
 void cg_r_b(dwf_ctx *c, T *r, const T *rin, const T *w, int base, int stride, int izz, int iww, int64_t n, int nrhs) {
     dim3 g = grid_b<T>(c, n, nrhs, 16);
-    cg_r_b_kernel<T><<<g, BT, 0, c->stream>>>(r, rin, w, c->scal.as<double>(), base, stride, izz, iww, n);
+    launch_after(cg_r_b_kernel<T>, g, dim3(BT), 0, c->stream, r, rin, w, c->scal.as<double>(), base, stride, izz, iww, n);
+    DWF_CHECK_LAUNCH();
+}
+
+template <typename T>
+void cg_p_b(dwf_ctx *c, T *pout, const T *pin, const T *z, int base, int stride, int izz, int inew, int64_t n, int nrhs) {
+    dim3 g = grid_b<T>(c, n, nrhs, 16);
+    launch_after(cg_p_b_kernel<T>, g, dim3(BT), 0, c->stream, pout, pin, z, c->scal.as<double>(), base, stride, izz, inew, n);
     DWF_CHECK_LAUNCH();
 }
 
@@ -548,13 +586,14 @@ template <typename T> void combo_b(dwf_ctx *c, T *x, T *const *V, int k, const d
 }
 
 template <typename T>
-void cg_combine_b(dwf_ctx *c, T *x, T *const *Z, int k, int base, int stride, int zb, int wb, int64_t n, int nrhs) {
-    DWF_REQUIRE(k >= 1 && k <= 32, DWF_EINVAL, "cg_combine_b: 1 to 32 stored residuals");
+void cg_combine_b(dwf_ctx *c, T *x, T *const *Z, int k, int base, int stride, int zb, int wb, bool directions, int64_t n,
+                  int nrhs) {
+    DWF_REQUIRE(k >= 1 && k <= 32, DWF_EINVAL, "cg_combine_b: 1 to 32 stored fields");
     dim3 gr = grid_b<T>(c, n, nrhs, 16);
     MArgs<T> a;
     a.k = k;
     for (int j = 0; j < k; ++j) a.v[j] = Z[j];
-    cg_combine_b_kernel<T><<<gr, BT, 0, c->stream>>>(x, a, c->scal.as<double>(), base, stride, zb, wb, n);
+    cg_combine_b_kernel<T><<<gr, BT, 0, c->stream>>>(x, a, c->scal.as<double>(), base, stride, zb, wb, directions ? 1 : 0, n);
     DWF_CHECK_LAUNCH();
 }
 
@@ -582,11 +621,12 @@ void cg_redirect(dwf_ctx *c, T *p, const T *zt, const T *z, int izt, int iz, int
     template void multidot_b<T>(dwf_ctx *, BatchScratch &, int, int, T *const *, int, const T *, int64_t, int); \
     template void multiaxpy_b<T>(dwf_ctx *, T *, T *const *, int, int, int, double, int64_t, int);            \
     template void cg_r_b<T>(dwf_ctx *, T *, const T *, const T *, int, int, int, int, int64_t, int);          \
+    template void cg_p_b<T>(dwf_ctx *, T *, const T *, const T *, int, int, int, int, int64_t, int);          \
     template void cg_px_b<T>(dwf_ctx *, T *, T *, const T *, const T *, int, int, int, int, int, int64_t, int, bool, \
                              bool);                                                                            \
     template void cg_pxd_b<T>(dwf_ctx *, T *, T *, const T *, T *const *, int, const T *, int, int, int, int, int, \
                               int, int64_t, int, int);                                                         \
-    template void cg_combine_b<T>(dwf_ctx *, T *, T *const *, int, int, int, int, int, int64_t, int);        \
+    template void cg_combine_b<T>(dwf_ctx *, T *, T *const *, int, int, int, int, int, bool, int64_t, int);  \
     template void cg_chunk_b<T>(dwf_ctx *, T *, T *, T *const *, int, bool, bool, int, int, int, int, int, int,   \
                                 int64_t, int);                                                                 \
     template void normalised_b<T>(dwf_ctx *, double2 *, const T *, int, int, int64_t, int);                   \

@@ -60,14 +60,14 @@ __device__ __forceinline__ void hop_row(C<R> acc[12], const C<R> *p, int ls_rt, 
 // instructions per 5D site, 3.0 ms of the pipe at 16^3 x 32 x 16.  With the
 // complex multiply-add as four fused instructions 3.37 ms; as six 4.66 ms.
 // 168 registers and 3 CTAs per SM instead of 128 and 4 measured the same.
-// EPI 0 .. 4: the epilogues of the paired FP32 kernel (dslash_pair.cuh), here
-// for FP64: nothing, |out|^2, z - a D^+ in, z - D in, D in + a z (EPI > 0 runs
-// whole warps: blockDim.x a multiple of 32, no early exit before the norms).
+// EPI 0, 1, 3: the epilogues of the paired FP32 kernel (dslash_pair.cuh) that
+// FP64 uses as well: nothing, |out|^2, zin - D in (EPI > 0 runs whole warps:
+// blockDim.x a multiple of 32, no early exit before the norms).
 template <typename R, bool DAG, bool SHFL, int LS, int MINB, int EPI>
 __global__ void __launch_bounds__(128, MINB)
 dslash_kernel(C<R> *out, const C<R> *in, const C<R> *__restrict__ U, Geom g, R diag, R mf,
-              int spb, int64_t field, NormOut nout, ZUpdateT<R> zu) {
-    constexpr bool NORM = EPI == 1 || EPI == 2 || EPI == 4;
+              int spb, int64_t field, NormOut nout, const C<R> *zin) {
+    constexpr bool NORM = EPI == 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C<R> *sU = reinterpret_cast<C<R> *>(smem_raw);               // [spb][8][10] (9 used)
     int *sN = reinterpret_cast<int *>(sU + (size_t)spb * 80);       // [spb][8]
@@ -109,8 +109,8 @@ dslash_kernel(C<R> *out, const C<R> *in, const C<R> *__restrict__ U, Geom g, R d
     if (!SHFL && !NORM && !active) return;
     const int row = 12 * Ls;
     C<R> acc[12], self[12];
-    if (EPI >= 2 && active) {  // the second field, into L2 ahead of its use
-        const C<R> *zp = zu.zin + rhs_off + (size_t)site * row + s;
+    if (EPI == 3 && active) {  // the second field, into L2 ahead of its use
+        const C<R> *zp = zin + rhs_off + (size_t)site * row + s;
 #pragma unroll
         for (int k = 0; k < 12; ++k) asm volatile("prefetch.global.L2 [%0];\n" ::"l"(zp + k * Ls));
     }
@@ -174,24 +174,11 @@ dslash_kernel(C<R> *out, const C<R> *in, const C<R> *__restrict__ U, Geom g, R d
         hop_row<3, true, R, LS>(acc, in + (size_t)sNs[7] * row + s, Ls, sUs + 7 * 10, -fs);
         pdl_dependents();
         C<R> *o = out + (size_t)site * row + s;
-        R a = R(1);
-        if (EPI == 2 || EPI == 4) {
-            const double ww = zu.ww[(size_t)blockIdx.y * zu.stride];
-            a = ww > 0.0 ? (R)(zu.zz[(size_t)blockIdx.y * zu.stride] / ww) : R(0);
-        }
-        const C<R> *zp = EPI >= 2 ? zu.zin + rhs_off + (size_t)site * row + s : nullptr;
+        const C<R> *zp = EPI == 3 ? zin + rhs_off + (size_t)site * row + s : nullptr;
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
             C<R> v = acc[k];
-            if (EPI == 2 || EPI == 3) {
-                const C<R> z = zp[k * Ls];
-                v.x = z.x - a * v.x;
-                v.y = z.y - a * v.y;
-            } else if (EPI == 4) {
-                const C<R> z = zp[k * Ls];
-                v.x += a * z.x;
-                v.y += a * z.y;
-            }
+            if (EPI == 3) v = zp[k * Ls] - v;
             o[k * Ls] = v;
             if (NORM) {
                 nrm += v.x * v.x;
@@ -209,7 +196,7 @@ dslash_kernel(C<R> *out, const C<R> *in, const C<R> *__restrict__ U, Geom g, R d
 
 template <typename R, int EPI>
 void launch(dwf_ctx *c, C<R> *out, const C<R> *in, const C<R> *U, bool dag, int nrhs, double *nslot = nullptr,
-            int nstride = 0, const ZUpdateT<R> *zu = nullptr) {
+            int nstride = 0, const C<R> *zin = nullptr) {
     const Geom &g = c->g;
     DWF_REQUIRE(g.V * g.Ls * 12 < (int64_t)1 << 31 && g.V < (int64_t)1 << 31, DWF_EINVAL,
                 "lattice too large for 32-bit element offsets of one field");
@@ -232,7 +219,6 @@ void launch(dwf_ctx *c, C<R> *out, const C<R> *in, const C<R> *U, bool dag, int 
     int64_t field = g.V * g.Ls * 12;
     R diag = R(5.0 - c->M5), mf = R(c->mf);
     const NormOut nout = nslot ? norm_out(c, grid, nrhs, nslot, nstride) : NormOut{};
-    const ZUpdateT<R> z = zu ? *zu : ZUpdateT<R>{};
     // register budget: 8 CTAs/SM (64 registers, small spills) or 6 (80);
     // DWF_DSLASH_MINB=6 selects the latter
     static const int minb = [] {
@@ -241,18 +227,17 @@ void launch(dwf_ctx *c, C<R> *out, const C<R> *in, const C<R> *U, bool dag, int 
     }();
 #define DLM(D, S, L, M)                                                                                             \
     launch_after(dslash_kernel<R, D, S, L, M, EPI>, grid, dim3(threads), smem, c->stream, out, in, U, g, diag, mf, spb, \
-                 field, nout, z)
+                 field, nout, zin)
 #define DL(D, S, L)                                          \
     do {                                                     \
         if constexpr (sizeof(R) == 8) DLM(D, S, L, 4);       \
         else if (minb == 6) DLM(D, S, L, 6);                 \
         else DLM(D, S, L, 8);                                \
     } while (0)
-    // (EPI 2 is a D^+ kernel, 3 and 4 are D kernels; the others come in both)
+    // (EPI 3 is a D kernel; the others come in both)
 #define DLD(S, L)                                            \
     do {                                                     \
-        if constexpr (EPI == 2) DL(true, S, L);              \
-        else if constexpr (EPI > 2) DL(false, S, L);         \
+        if constexpr (EPI == 3) DL(false, S, L);             \
         else if (dag) DL(true, S, L);                        \
         else DL(false, S, L);                                \
     } while (0)
@@ -370,28 +355,7 @@ void dslash_norm(dwf_ctx *c, double2 *out, const double2 *in, bool dag, int nrhs
 void dslash_residual(dwf_ctx *c, double2 *res, const double2 *x, const double2 *b, int nrhs) {
     DWF_REQUIRE(res != x && res != b, DWF_EINVAL, "residual: output must not alias an input");
     ProfScope ps(c, K_DSLASH_F64, nrhs);
-    const ZUpdateT<double> zu{b, nullptr, nullptr, 0, 0};
-    launch<double, 3>(c, res, x, c->U64.as<double2>(), false, nrhs, nullptr, 0, &zu);
-    c->applies64 += nrhs;
-}
-
-void dslash_wupdate(dwf_ctx *c, double2 *wout, const double2 *z, const double2 *win, int nrhs, int slot, int stride,
-                    int inum, int iden) {
-    DWF_REQUIRE(wout != win && wout != z, DWF_EINVAL, "direction update: output must not alias an input");
-    ProfScope ps(c, K_DSLASH_F64, nrhs);
-    double *s = c->scal.as<double>();
-    const ZUpdateT<double> zu{win, s + inum, s + iden, stride, 1};
-    launch<double, 4>(c, wout, z, c->U64.as<double2>(), false, nrhs, s + slot, stride, &zu);
-    c->applies64 += nrhs;
-}
-
-void dslash_zupdate(dwf_ctx *c, double2 *zout, const double2 *w, const double2 *zin, int nrhs, int slot, int stride,
-                    int izz, int iww) {
-    DWF_REQUIRE(zout != zin && zout != w, DWF_EINVAL, "residual update: output must not alias an input");
-    ProfScope ps(c, K_DSLASH_F64, nrhs);
-    double *s = c->scal.as<double>();
-    const ZUpdateT<double> zu{zin, s + izz, s + iww, stride, 0};
-    launch<double, 2>(c, zout, w, c->U64.as<double2>(), true, nrhs, s + slot, stride, &zu);
+    launch<double, 3>(c, res, x, c->U64.as<double2>(), false, nrhs, nullptr, 0, b);
     c->applies64 += nrhs;
 }
 

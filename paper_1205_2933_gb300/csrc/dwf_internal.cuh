@@ -213,15 +213,14 @@ inline Brick pick_brick(const Geom &g, int sites) {
 
 // The normal-equations residual update of CGNR, z <- z - a D^+ w, with
 // a = zz / ww of each right-hand side read from the scalar slots.
-template <typename R> struct ZUpdateT {
-    const C<R> *zin;    // the second field (not the output buffer)
+struct ZUpdate {
+    const float2 *zin;  // the second field (not the output buffer)
     const double *zz;   // numerator of a for right-hand side r at zz[r * stride]
     const double *ww;   // denominator of a at ww[r * stride]
     int stride;
     int add;            // 1: out = D in + a zin (EPI 4); 0: out = zin - a D^+ in (EPI 2)
     int stream;         // paired kernel: zin and out leave L2 first
 };
-using ZUpdate = ZUpdateT<float>;
 
 // fifth extents of the paired FP32 Dslash, and its sites per warp there
 inline bool dslash_pair_supported(int Ls) {
@@ -343,15 +342,11 @@ void dslash_residual(dwf_ctx *c, float2 *res, const float2 *x, const float2 *b, 
 // CGNR's w = D p carried without p: w_out = D z + b w_in for every right-hand
 // side r, b = scal[inum + r stride] / scal[iden + r stride], and |w_out|^2 into
 // scal[slot + r stride] (when dslash_norm_fused(c))
-void dslash_wupdate(dwf_ctx *c, double2 *wout, const double2 *z, const double2 *win, int nrhs, int slot, int stride,
-                    int inum, int iden);
 void dslash_wupdate(dwf_ctx *c, float2 *wout, const float2 *z, const float2 *win, int nrhs, int slot, int stride,
                     int inum, int iden);
 // CGNR's normal-equations residual update z_out = z_in - a D^+ w for every
 // right-hand side r, a = scal[izz + r stride] / scal[iww + r stride], and
 // |z_out|^2 into scal[slot + r stride] (available when dslash_norm_fused(c))
-void dslash_zupdate(dwf_ctx *c, double2 *zout, const double2 *w, const double2 *zin, int nrhs, int slot, int stride,
-                    int izz, int iww);
 void dslash_zupdate(dwf_ctx *c, float2 *zout, const float2 *w, const float2 *zin, int nrhs, int slot, int stride,
                     int izz, int iww);
 

@@ -609,17 +609,26 @@ template <typename R> class Runner {
     }
 };
 
-// The setup's relaxation carries z by recursion at these fifth extents; at the
-// other ones it keeps r (z = D^+ r fresh), whose FP32 rounding in the vectors
-// is 2.5 times smaller (1.3e-6 against 3.1e-6 after 8 steps).
-bool relax_zform(int Ls) { return Ls == 4 || Ls == 8 || Ls == 16 || Ls == 32 || Ls == 64; }
+// Two forms of CGNR on several fields at once.  Either r is kept and z = D^+ r
+// formed afresh, with r and the direction p updated by kernels of their own; or
+// z and w = D p are carried by recursion in the Dslash epilogues, which saves
+// those passes over the fields and rounds 2.8 times worse, because what a step
+// rounds off z stays in it (FP32 V-cycle with 16 steps: 1.3e-7 against 3.7e-7 of
+// the result; 8 steps of the relaxation: 1.3e-6 against 3.2e-6 of the vectors).
+// The carried form serves FP32 batches at the extents that leave no lane of the
+// paired Dslash's warps idle (Ls / 2 divides 32): theirs is the rounding that
+// callers of several sources have always had there, and keeping r would cost
+// them a third of their time (V-cycle of 12 fields, 12^3 x 16 x 16). One
+// right-hand side, FP64 and the other extents keep r, as they always did.
+bool carried_form(int Ls, int nr, bool f32) { return f32 && nr > 1 && Ls >= 4 && Ls % 2 == 0 && 32 % (Ls / 2) == 0; }
 
 // Batched solve: all right-hand sides advance together.  Fine-level kernels
 // run over the whole batch (the Dslash with nrhs in its grid, the basis of
 // the transfers read once per 12 right-hand sides); every right-hand side
 // keeps its own GCR coefficients, triangular transform and convergence
 // state, and stops changing once converged.  Coarsest-level solves run per
-// right-hand side through the fused kernel.  FP32 V-cycle, 2 levels, nu_1 = 0.
+// right-hand side through the fused kernel.  FP32 or (one right-hand side at a
+// time) FP64 V-cycle, 2 levels, nu_1 = 0.
 template <typename R> class BatchRunner {
   public:
     using T = C<R>;
@@ -706,8 +715,8 @@ template <typename R> class BatchRunner {
 
     static constexpr int CHUNK = 8;  // iterations per chunk of a long CGNR run in the residual-keeping form
 
-    // whether the smoother may keep its nu residuals (nu fields per right-hand
-    // side at workspace indices 100 ..): decided once per runner and nu;
+    // whether the smoother may keep its nu residuals or directions (nu fields per
+    // right-hand side at workspace indices 100 ..): decided once per runner and nu;
     // DWF_SMOOTHER_HISTORY=0 in the environment selects the other form
     int hist_nu_ = -1;
     bool hist_ok_ = false;
@@ -741,9 +750,29 @@ template <typename R> class BatchRunner {
         }
         // the Dslash can produce the norms of its outputs in its epilogue
         const bool fused = fused_ok();
+        const bool carry = fused && carried_form(c->g.Ls, nr, std::is_same<R, float>::value);
         T *w = wsb(0, 3);
-        {
-            if (fused && accumulate && rtol <= 0.0 && iters <= 32 && keep_history(iters)) {
+        if (fused && !carry && accumulate && rtol <= 0.0 && iters <= 32 && keep_history(iters)) {
+            // The smoother that keeps r, when its directions p_0 .. p_{nu-1} fit in
+            // memory: x gains sum_k a_k p_k once at the end, in the order of the
+            // steps, instead of one read and write of x per iteration
+            constexpr int ZB = 8, WB = 72;  // slots of |z_k|^2 and |w_k|^2
+            std::vector<T *> P(iters);
+            for (int j = 0; j < iters; ++j) P[j] = wsb(0, 100 + j);
+            T *r = wsb(0, 0), *z = wsb(0, 1);
+            dslash_norm(c, P[0], b, true, nr, SB + ZB, SS);  // p_0 = z_0 = D^+ r_0, r_0 = b
+            for (int k = 0;; ++k) {
+                dslash_norm(c, w, P[k], false, nr, SB + WB + k, SS);
+                if (k + 1 == iters) break;
+                cg_r_b<T>(c, r, k == 0 ? b : r, w, SB, SS, ZB + k, WB + k, N, nr);
+                dslash_norm(c, z, r, true, nr, SB + ZB + k + 1, SS);
+                cg_p_b<T>(c, P[k + 1], P[k], z, SB, SS, ZB + k, ZB + k + 1, N, nr);
+            }
+            cg_combine_b<T>(c, x, P.data(), iters, SB, SS, ZB, WB, true, N, nr);
+            return;
+        }
+        if constexpr (std::is_same<R, float>::value) {
+            if (carry && accumulate && rtol <= 0.0 && iters <= 32 && keep_history(iters)) {
                 // The smoother's form when its residuals z_0 .. z_{nu-1} fit in
                 // memory: no direction p and no per-iteration solution update.
                 // w = D p follows w_{k+1} = D z_{k+1} + b_k w_k (p_{k+1} = z_{k+1}
@@ -764,10 +793,10 @@ template <typename R> class BatchRunner {
                     dslash_wupdate(c, wb[(k + 1) & 1], Zh[k + 1], wb[k & 1], nr, SB + WB + k + 1, SS, SB + ZB + k + 1,
                                    SB + ZB + k);
                 }
-                cg_combine_b<T>(c, x, Zh.data(), iters, SB, SS, ZB, WB, N, nr);
+                cg_combine_b<T>(c, x, Zh.data(), iters, SB, SS, ZB, WB, false, N, nr);
                 return;
             }
-            if (fused && !accumulate && relax_zform(c->g.Ls) && keep_history(CHUNK + 1)) {
+            if (carry && !accumulate && keep_history(CHUNK + 1)) {
                 // A long run (the setup's relaxation) in the same form, in
                 // chunks of CHUNK iterations: each keeps its residuals in a ring
                 // of CHUNK + 1 buffers, and its end adds sum a_k p_k to x and
@@ -836,8 +865,8 @@ template <typename R> class BatchRunner {
             read_block(sv);
             for (int q = 0; q < nr; ++q) r0[q] = std::sqrt(sv[(size_t)q * SS + irr]);
         }
-        {
-            if (fused && (accumulate ? rtol <= 0.0 : relax_zform(c->g.Ls))) {
+        if constexpr (std::is_same<R, float>::value) {
+            if (carry && !(accumulate && rtol > 0.0)) {
                 // r itself is never needed: the normal-equations residual
                 // z = D^+ r follows its own recursion z <- z - a D^+ w (the
                 // same iterates in exact arithmetic), which the D^+ Dslash
@@ -1643,7 +1672,7 @@ static void keep_buffers(MGState &mg, MGState &old) {
     if (!f32 || !batch_on() || L.nadapt < 2 || L.nadapt > 32 || mg.p.setup_iters0 < 1) return;
     // the workspaces of relax and of cgnr_b's form at this fifth extent
     std::vector<int> used = {0, 2, 3, 8, 9, 10};
-    if (relax_zform(L.lg.g.Ls)) {
+    if (carried_form(L.lg.g.Ls, L.nadapt, f32)) {
         used.push_back(13);
         for (int j = 0; j <= 8; ++j) used.push_back(100 + j);
     } else {

@@ -165,6 +165,9 @@ template <typename T> void multiaxpy_b(dwf_ctx *c, T *w, T *const *V, int k, int
 // r = rin - a w (rin may be r), a = |z|^2 / |w|^2 from the slots
 template <typename T>
 void cg_r_b(dwf_ctx *c, T *r, const T *rin, const T *w, int base, int stride, int izz, int iww, int64_t n, int nrhs);
+// pout = z + beta pin (pin may be pout), beta = |z'|^2 / |z|^2 from the slots inew, izz
+template <typename T>
+void cg_p_b(dwf_ctx *c, T *pout, const T *pin, const T *z, int base, int stride, int izz, int inew, int64_t n, int nrhs);
 // x += a pin (x = a pin with xinit); unless last, pout = z + beta pin (pin may be pout)
 template <typename T>
 void cg_px_b(dwf_ctx *c, T *x, T *pout, const T *pin, const T *z, int base, int stride, int izz, int iww, int inew,
@@ -178,10 +181,12 @@ template <typename T>
 void cg_pxd_b(dwf_ctx *c, T *x, T *pout, const T *pin, T *const *pend, int np, const T *z, int base, int stride,
               int izz, int iww, int inew, int ia, int64_t n, int nrhs, int mode);
 // x += the solution of k CGNR iterations expressed in their stored
-// normal-equations residuals Z[0..k-1] (k <= 32); |z_j|^2 in slot zb + j and
-// |w_j|^2 = |D p_j|^2 in slot wb + j of each right-hand side's block
+// normal-equations residuals Z[0..k-1] (k <= 32), or with `directions` in their
+// stored directions p_j = Z[j]; |z_j|^2 in slot zb + j and |w_j|^2 = |D p_j|^2
+// in slot wb + j of each right-hand side's block
 template <typename T>
-void cg_combine_b(dwf_ctx *c, T *x, T *const *Z, int k, int base, int stride, int zb, int wb, int64_t n, int nrhs);
+void cg_combine_b(dwf_ctx *c, T *x, T *const *Z, int k, int base, int stride, int zb, int wb, bool directions, int64_t n,
+                  int nrhs);
 // End of a chunk of m CGNR iterations from k0 that kept their residuals
 // Z[t-1] = z_{k0+t} (t = 1 .. m-1, and m with next): x (+)= sum_t a_t p_t with
 // p the chunk's first direction, and with next p <- the next chunk's first
