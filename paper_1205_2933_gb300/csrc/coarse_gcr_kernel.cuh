@@ -328,14 +328,31 @@ template <typename R, typename LT, int NV, int NPTS> struct SmemPlan {
     }
 };
 
+// the sum of N values (a power of two) in pairs
+template <int N, typename T> __device__ __forceinline__ T pair_sum(const T (&v)[N]) {
+    T t[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) t[i] = v[i];
+#pragma unroll
+    for (int h = N / 2; h >= 1; h /= 2)
+#pragma unroll
+        for (int i = 0; i < h; ++i) t[i] = t[i] + t[i + h];
+    return t[0];
+}
+
 template <typename R, typename LT, int NV> __device__ __forceinline__ C<R> row_times(const unsigned char *row, const C<R> *x) {
-    // NV links of one row in accesses of 16 bytes (8 where the row is no multiple)
+    // NV links of one row in accesses of 16 bytes (8 where the row is no multiple),
+    // summed in several chains of at most four links: one chain of 24 rounds 1.4
+    // times worse than the warp-wide sum of the kernel above
+    constexpr int NA = NV % 8 == 0 ? 8 : NV % 4 == 0 ? 4 : 2;
     constexpr int B = NV * sizeof(LT) % 16 == 0 ? 16 : 8;
     constexpr int E = B / (int)sizeof(LT) > 0 ? B / (int)sizeof(LT) : 1;
     struct alignas(B) Chunk {
         LT e[E];
     };
-    C<R> acc = mk<R>(0, 0);
+    C<R> acc[NA];
+#pragma unroll
+    for (int i = 0; i < NA; ++i) acc[i] = mk<R>(0, 0);
     constexpr int NCH = NV / E;
     Chunk ch[NCH < 8 ? NCH : 8];
 #pragma unroll
@@ -348,9 +365,9 @@ template <typename R, typename LT, int NV> __device__ __forceinline__ C<R> row_t
             if (c0 + i < NCH)
 #pragma unroll
                 for (int j = 0; j < E; ++j)
-                    cfma(acc, LRead<LT>::template get<R>(ch[i].e, j), x[(c0 + i) * E + j]);
+                    cfma(acc[((c0 + i) * E + j) % NA], LRead<LT>::template get<R>(ch[i].e, j), x[(c0 + i) * E + j]);
     }
-    return acc;
+    return pair_sum<NA>(acc);
 }
 
 // The same GCR, with what a CTA owns of every vector (the directions Z and W,
@@ -360,8 +377,9 @@ template <typename R, typename LT, int NV> __device__ __forceinline__ C<R> row_t
 // for the reduction.  The products <W_i, w>, |w|^2 and <w, r> are reduced
 // together: with W orthonormal |w|^2 loses sum |<W_i, w>|^2 in the projection
 // and <w, r> does not change (r is orthogonal to the W_i).  Where the
-// projection took 3/4 or more of |w|^2, where that difference would lose
-// digits, a second one follows with a reduction of its own.  The stencil: one
+// projection took 1 % or more of |w|^2, where that difference and the W_i's
+// rounding would lose digits, a second one follows with a reduction of its own
+// (always taking two rounds no better).  The stencil: one
 // thread per (direction, row) of a site, the neighbours' values staged.
 // Bound by the latency of the two barriers and of one L2 round trip after
 // each: 512 sites x 24 in BF16 44 us where the vectors in global memory, four
@@ -409,10 +427,13 @@ __global__ void __launch_bounds__(CT) coarse_gcr_smem_kernel(Args<R, LT> a, int 
         __syncthreads();
         for (int e = tid; e < own; e += CT) {
             const int site = e / NV, k = e - site * NV;
-            C<R> v = sp[site * NPTS * NV + k];
+            C<R> t[4];
 #pragma unroll
-            for (int d = 1; d < NPTS; ++d) v = v + sp[(site * NPTS + d) * NV + k];
-            dst[e] = v;
+            for (int d = 0; d < NPTS - 1; ++d) {
+                const C<R> v = sp[(site * NPTS + d + 1) * NV + k];
+                t[d % 4] = d < 4 ? v : t[d % 4] + v;
+            }
+            dst[e] = sp[site * NPTS * NV + k] + pair_sum<4>(t);
         }
         __syncthreads();
     };
@@ -512,14 +533,14 @@ __global__ void __launch_bounds__(CT) coarse_gcr_smem_kernel(Args<R, LT> a, int 
                     C<R> wv = w[e], zv = z[e];
                     for (int i = 0; i < k; ++i) {
                         const C<R> m = mk<R>(-(R)tot[i].x, -(R)tot[i].y);
-                        cfma(wv, m, W(i)[e]);
-                        cfma(zv, m, Z(i)[e]);
+                        cadd_prod(wv, m, W(i)[e]);
+                        cadd_prod(zv, m, Z(i)[e]);
                     }
                     w[e] = wv;
                     z[e] = zv;
                 }
                 __syncthreads();  // tot is rewritten by the next reduction
-                const bool again = pass == 0 && removed >= 0.75 * ww;
+                const bool again = pass == 0 && removed >= 0.01 * ww;
                 ww -= removed;
                 if (!again) break;
             }
@@ -530,8 +551,8 @@ __global__ void __launch_bounds__(CT) coarse_gcr_smem_kernel(Args<R, LT> a, int 
             for (int e = tid; e < own; e += CT) {
                 const C<R> zv = sc * z[e], wv = sc * w[e];
                 C<R> xv = x[e], rv = r[e];
-                cfma(xv, al, zv);
-                cfma(rv, mal, wv);
+                cadd_prod(xv, al, zv);
+                cadd_prod(rv, mal, wv);
                 z[e] = zv;
                 w[e] = wv;
                 x[e] = xv;

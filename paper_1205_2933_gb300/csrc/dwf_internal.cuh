@@ -57,6 +57,14 @@ template <typename T> __host__ __device__ __forceinline__ void cfmac(T &acc, T a
     acc.y -= a.y * b.x;
 }
 
+// acc += a * b with the product formed on its own: six instructions, of which
+// one rounds at the size of acc where each of cfma's four does.  For vector
+// updates, whose products are small against what they are added to.
+template <typename T> __host__ __device__ __forceinline__ void cadd_prod(T &acc, T a, T b) {
+    acc.x += a.x * b.x - a.y * b.y;
+    acc.y += a.x * b.y + a.y * b.x;
+}
+
 template <typename TO, typename TI> __host__ __device__ __forceinline__ TO cvt(TI a);
 template <> __host__ __device__ __forceinline__ double2 cvt<double2, double2>(double2 a) { return a; }
 template <> __host__ __device__ __forceinline__ float2 cvt<float2, float2>(float2 a) { return a; }

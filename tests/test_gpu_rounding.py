@@ -64,3 +64,59 @@ def test_fp32_vcycle(G, dims, Ls, nu, nrhs, bound):
         torch.cuda.synchronize()
         ctx.close()
     assert _rel(out[1], out[0]) < bound
+
+
+def _gcr64(Y, dims, b, its, restart):
+    """GCR of the coarse stencil Y [V][9][n][n] in FP64, its directions orthogonalised twice."""
+    V, n = Y.shape[0], Y.shape[2]
+    site = torch.arange(V, device="cuda").reshape(tuple(dims)[::-1])
+    nb = [site.reshape(-1)]
+    for mu in range(4):
+        nb += [torch.roll(site, s, 3 - mu).reshape(-1) for s in (-1, 1)]
+
+    def A(v):
+        v = v.reshape(V, n)
+        return sum(torch.einsum("skl,sl->sk", Y[:, d], v[nb[d]]) for d in range(9)).reshape(-1)
+
+    x, r, Z, W = torch.zeros_like(b), b.clone(), [], []
+    for _ in range(its):
+        z, w = r.clone(), A(r)
+        for zi, wi in 2 * list(zip(Z, W)):
+            c = torch.vdot(wi, w)
+            w, z = w - c * wi, z - c * zi
+        nw = w.norm()
+        Z.append(z / nw)
+        W.append(w / nw)
+        a = torch.vdot(W[-1], r)
+        x, r = x + a * Z[-1], r - a * W[-1]
+        if len(Z) == restart:
+            r, Z, W = b - A(x), [], []
+    return x
+
+
+@pytest.mark.parametrize("prec", [0, 1], ids=["f64", "f32"])
+@pytest.mark.parametrize("dims,Ls,nvec,block,restart,its,f32,f64",
+                         [((8, 8, 8, 8), 4, 8, (2, 2, 2, 2), 16, 12, 1.36, 3.3), ((8, 8, 8, 8), 4, 16, (2, 2, 2, 2), 16, 32, 1.53, 4.1),
+                          ((6, 6, 3, 6), 4, 24, (1, 1, 1, 1), 16, 16, 1.37, 3.6),
+                          ((8, 8, 8, 8), 8, 24, (4, 4, 2, 2), 16, 24, 1.44, 3.8)])
+def test_coarsest_gcr(G, dims, Ls, nvec, block, restart, its, f32, f64, prec):
+    """A fixed number of coarsest GCR iterations against FP64 on the same links.
+    f32 (1e-7), f64 (1e-16): what the solver with FP64 sums, two projections each
+    and warp-wide stencil sums leaves; 15 % between one shape's right-hand sides."""
+    ctx = _ctx(dims, Ls)
+    p = M._params(G, setup_iters0=30, setup_sweeps=0, smoother_prec=prec, coarse_prec=[prec], coarsest_tol=0.0,
+                  coarsest_maxiter=its, coarse_restart=restart)
+    G.mg_setup(ctx.h, 2, [nvec], [block], p, torch.from_numpy(I.random_vectors(nvec // 2, dims, Ls, 3)).cuda())
+    d, n = G.mg_level_info(ctx.h, 1)
+    V, dt = int(np.prod(d)), torch.complex64 if prec else torch.complex128
+    y = torch.empty(V * 9 * n * n, dtype=torch.complex128, device="cuda")
+    G.mg_get_coarse_links(ctx.h, 1, y)
+    Y = y.to(dt).to(torch.complex128).reshape(V, 9, n, n)
+    err = 0.0
+    for s in range(4):
+        b = _randn(V * n, 7 + s, dt)
+        x = torch.empty_like(b)
+        G.mg_coarse_solve(ctx.h, 1, x, b)
+        err += _rel(x, _gcr64(Y, d, b.to(torch.complex128), its, restart)) / 4
+    assert err < 1.15 * (f32 * 1e-7 if prec else f64 * 1e-16)
+    ctx.close()
