@@ -13,7 +13,10 @@ constexpr int RED_THREADS = 256;
 constexpr int RED_MAX_BLOCKS = 1024;
 
 // Per-thread partial sums in the storage precision (FP32 FMAs for FP32
-// fields), combined across threads and CTAs in FP64.
+// fields), combined across threads and CTAs in FP64.  Fused multiply-adds, one
+// product each (the FP64 pipe bounds these loops), in two chains per sum: each
+// rounds at half the size of the whole, so that both together round no worse
+// than one chain of two products at a time.
 template <typename T> struct Acc;
 template <> struct Acc<double2> { using type = double; };
 template <> struct Acc<float2> { using type = float; };
@@ -22,16 +25,16 @@ template <typename TX, typename TY>
 __global__ void __launch_bounds__(RED_THREADS) dot_kernel(const TX *__restrict__ x, const TY *__restrict__ y, int64_t n,
                                                           double *part, unsigned *count, double *out) {
     using A = typename Acc<TX>::type;
-    A ar = 0, ai = 0;
+    A ar[2] = {0, 0}, ai[2] = {0, 0};
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         TX u = x[i];
         TY v = y[i];
-        ar += (A)u.x * (A)v.x;  // one product at a time: fused multiply-adds (the FP64 pipe bounds these loops)
-        ai += (A)u.x * (A)v.y;
-        ar += (A)u.y * (A)v.y;
-        ai -= (A)u.y * (A)v.x;
+        ar[0] += (A)u.x * (A)v.x;
+        ai[0] += (A)u.x * (A)v.y;
+        ar[1] += (A)u.y * (A)v.y;
+        ai[1] -= (A)u.y * (A)v.x;
     }
-    const double m[2] = {(double)ar, (double)ai};
+    const double m[2] = {(double)(ar[0] + ar[1]), (double)(ai[0] + ai[1])};
     grid_sums<2>(m, part, count, out, 2);
 }
 
@@ -39,13 +42,13 @@ template <typename T>
 __global__ void __launch_bounds__(RED_THREADS) norm2_kernel(const T *__restrict__ x, int64_t n, double *part,
                                                             unsigned *count, double *out) {
     using A = typename Acc<T>::type;
-    A a = 0;
+    A a[2] = {0, 0};
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         T u = x[i];
-        a += (A)u.x * (A)u.x;
-        a += (A)u.y * (A)u.y;
+        a[0] += (A)u.x * (A)u.x;
+        a[1] += (A)u.y * (A)u.y;
     }
-    const double m[1] = {(double)a};
+    const double m[1] = {(double)(a[0] + a[1])};
     grid_sums<1>(m, part, count, out, 1);
 }
 
@@ -58,25 +61,25 @@ template <typename T, int K>
 __global__ void __launch_bounds__(RED_THREADS) multidot_kernel(MultiDotArgs<T, K> a, const T *__restrict__ w, int64_t n,
                                                                double *part, unsigned *count, double *out) {
     using A = typename Acc<T>::type;
-    A ar[K], ai[K];
+    A ar[K][2], ai[K][2];
 #pragma unroll
-    for (int j = 0; j < K; ++j) ar[j] = ai[j] = 0;
+    for (int j = 0; j < K; ++j) ar[j][0] = ar[j][1] = ai[j][0] = ai[j][1] = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         T y = w[i];
 #pragma unroll
         for (int j = 0; j < K; ++j) {
             T u = a.v[j][i];
-            ar[j] += (A)u.x * (A)y.x;
-            ai[j] += (A)u.x * (A)y.y;
-            ar[j] += (A)u.y * (A)y.y;
-            ai[j] -= (A)u.y * (A)y.x;
+            ar[j][0] += (A)u.x * (A)y.x;
+            ai[j][0] += (A)u.x * (A)y.y;
+            ar[j][1] += (A)u.y * (A)y.y;
+            ai[j][1] -= (A)u.y * (A)y.x;
         }
     }
     double m[2 * K];
 #pragma unroll
     for (int j = 0; j < K; ++j) {
-        m[2 * j] = (double)ar[j];
-        m[2 * j + 1] = (double)ai[j];
+        m[2 * j] = (double)(ar[j][0] + ar[j][1]);
+        m[2 * j + 1] = (double)(ai[j][0] + ai[j][1]);
     }
     grid_sums<2 * K>(m, part, count, out, 2 * K);
 }

@@ -18,10 +18,12 @@ __global__ void caxpy_kernel(T *__restrict__ y, double2 ad, const T *__restrict_
     const R ar = (R)ad.x, ai = (R)ad.y;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         T xv = x[i], yv = y[i];
-        yv.x += ar * xv.x;
-        yv.y += ar * xv.y;
-        yv.x -= ai * xv.y;
-        yv.y += ai * xv.x;
+        if (ai == R(0)) {  // (most callers: half the FP64 operations)
+            yv.x += ar * xv.x;
+            yv.y += ar * xv.y;
+        } else {
+            cadd_prod(yv, mk<R>(ar, ai), xv);
+        }
         y[i] = yv;
     }
 }
@@ -129,16 +131,16 @@ __global__ void multiaxpy_dev_kernel(T *__restrict__ w, MultiArgs<T> a, const do
     }
     __syncthreads();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        T v = w[i];
+        T t{0, 0};  // small against w, which is rounded once
 #pragma unroll 8
         for (int j = 0; j < a.k; ++j) {
             T u = a.p[j][i];
-            v.x += cr[j] * u.x;
-            v.y += cr[j] * u.y;
-            v.x -= ci[j] * u.y;
-            v.y += ci[j] * u.x;
+            t.x += cr[j] * u.x;
+            t.y += cr[j] * u.y;
+            t.x -= ci[j] * u.y;
+            t.y += ci[j] * u.x;
         }
-        w[i] = v;
+        w[i] = w[i] + t;
     }
 }
 

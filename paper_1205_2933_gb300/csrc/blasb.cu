@@ -15,22 +15,25 @@ template <typename T> struct RealB;
 template <> struct RealB<float2> { using type = float; };
 template <> struct RealB<double2> { using type = double; };
 
+// Sums are kept in several chains, one per part of a product or more: a thread
+// adds up more elements than when every element had a CTA's share to itself, and
+// shorter chains at a fraction of the sum's size round no worse.
 // s[base + r*stride] = |x_r|^2
 template <typename T>
 __global__ void __launch_bounds__(BT) norm2_b_kernel(const T *__restrict__ x, int64_t n, double *part, unsigned *count,
                                                      double *s, int base, int stride) {
     using A = typename RealB<T>::type;
     x += (size_t)blockIdx.y * n;
-    A a = 0;
+    A a[2][2] = {{0, 0}, {0, 0}};
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n / Pack<T>::N; i += (int64_t)gridDim.x * blockDim.x) {
         const Pack<T> u = ldp(x, i);
 #pragma unroll
         for (int e = 0; e < Pack<T>::N; ++e) {
-            a += u.e[e].x * u.e[e].x;
-            a += u.e[e].y * u.e[e].y;
+            a[e][0] += u.e[e].x * u.e[e].x;
+            a[e][1] += u.e[e].y * u.e[e].y;
         }
     }
-    const double m[1] = {(double)a};
+    const double m[1] = {(double)((a[0][0] + a[0][1]) + (a[1][0] + a[1][1]))};
     grid_sums<1>(m, part + (size_t)blockIdx.y * gridDim.x, count + blockIdx.y, s + base + blockIdx.y * stride, 1);
 }
 
@@ -44,9 +47,9 @@ __global__ void __launch_bounds__(BT) multidot_b_kernel(VArgs<T, K> va, const T 
                                                         int stride) {
     using A = typename RealB<T>::type;
     const size_t off = (size_t)blockIdx.y * n;
-    A ar[K], ai[K];
+    A ar[K][2], ai[K][2];
 #pragma unroll
-    for (int j = 0; j < K; ++j) ar[j] = ai[j] = 0;
+    for (int j = 0; j < K; ++j) ar[j][0] = ar[j][1] = ai[j][0] = ai[j][1] = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n / Pack<T>::N; i += (int64_t)gridDim.x * blockDim.x) {
         const Pack<T> y = ldp(w + off, i);
         Pack<T> u[K];
@@ -56,17 +59,17 @@ __global__ void __launch_bounds__(BT) multidot_b_kernel(VArgs<T, K> va, const T 
         for (int j = 0; j < K; ++j)
 #pragma unroll
             for (int e = 0; e < Pack<T>::N; ++e) {
-                ar[j] += u[j].e[e].x * y.e[e].x;
-                ai[j] += u[j].e[e].x * y.e[e].y;
-                ar[j] += u[j].e[e].y * y.e[e].y;
-                ai[j] -= u[j].e[e].y * y.e[e].x;
+                ar[j][0] += u[j].e[e].x * y.e[e].x;
+                ai[j][0] += u[j].e[e].x * y.e[e].y;
+                ar[j][1] += u[j].e[e].y * y.e[e].y;
+                ai[j][1] -= u[j].e[e].y * y.e[e].x;
             }
     }
     double m[2 * K];
 #pragma unroll
     for (int j = 0; j < K; ++j) {
-        m[2 * j] = (double)ar[j];
-        m[2 * j + 1] = (double)ai[j];
+        m[2 * j] = (double)(ar[j][0] + ar[j][1]);
+        m[2 * j + 1] = (double)(ai[j][0] + ai[j][1]);
     }
     grid_sums<2 * K>(m, part + (size_t)blockIdx.y * 2 * K * gridDim.x, count + blockIdx.y,
                      s + base + blockIdx.y * stride, 2 * K);
@@ -90,18 +93,20 @@ __global__ void multiaxpy_b_kernel(T *__restrict__ w, MArgs<T> a, const double *
     }
     __syncthreads();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n / Pack<T>::N; i += (int64_t)gridDim.x * blockDim.x) {
-        Pack<T> v = ldp<T>(w + off, i);
+        Pack<T> v = ldp<T>(w + off, i), t{};
 #pragma unroll 8
         for (int j = 0; j < a.k; ++j) {
             const Pack<T> u = ldp(a.v[j] + off, i);
 #pragma unroll
             for (int e = 0; e < Pack<T>::N; ++e) {
-                v.e[e].x += cr[j] * u.e[e].x;
-                v.e[e].y += cr[j] * u.e[e].y;
-                v.e[e].x -= ci[j] * u.e[e].y;
-                v.e[e].y += ci[j] * u.e[e].x;
+                t.e[e].x += cr[j] * u.e[e].x;  // small against v, which is rounded once
+                t.e[e].y += cr[j] * u.e[e].y;
+                t.e[e].x -= ci[j] * u.e[e].y;
+                t.e[e].y += ci[j] * u.e[e].x;
             }
         }
+#pragma unroll
+        for (int e = 0; e < Pack<T>::N; ++e) v.e[e] = v.e[e] + t.e[e];
         stp(w + off, i, v);
     }
 }
@@ -289,10 +294,7 @@ __global__ void combo_b_kernel(T *__restrict__ x, MArgs<T> a, const double2 *__r
             const Pack<T> u = ldp(a.v[j] + off, i);
 #pragma unroll
             for (int e = 0; e < Pack<T>::N; ++e) {
-                v.e[e].x += cr[j] * u.e[e].x;
-                v.e[e].y += cr[j] * u.e[e].y;
-                v.e[e].x -= ci[j] * u.e[e].y;
-                v.e[e].y += ci[j] * u.e[e].x;
+                cadd_prod(v.e[e], mk<R>(cr[j], ci[j]), u.e[e]);
             }
         }
         stp(x + off, i, v);
