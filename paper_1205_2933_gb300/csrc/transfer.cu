@@ -55,8 +55,8 @@ __device__ __forceinline__ double2 piece(const double2 o[1]) { return o[0]; }
 
 // How a restriction CTA (8 warps) shares its work: RG groups of KG basis rows
 // times RC groups of NB right-hand sides times EH parts of the elements.  A
-// lane keeps KG x NB sums; KG NB is at most 36 (FP32) or 16 (FP64) for the
-// registers.  SE elements of all rows make one stage in shared memory.
+// lane keeps KG x NB sums; KG NB is at most 36 (FP32) or 8 (FP64, two chains
+// each) for the registers.  SE elements of all rows make one stage in shared memory.
 constexpr bool restrict_fits(int rg, int nv, int nb, int rc, int lim) {
     return nv % rg == 0 && (nv / rg) * nb <= lim && nv / rg <= 12 && rg * rc <= 8;
 }
@@ -66,7 +66,7 @@ constexpr int restrict_groups(int nv, int nb, int rc, int lim) {  // RG, or 0 wh
     return 0;
 }
 template <typename R, typename QT, int NV, int NB, int RC> struct RShape {
-    static constexpr int RG = restrict_groups(NV, NB, RC, sizeof(R) == 8 ? 16 : 36);
+    static constexpr int RG = restrict_groups(NV, NB, RC, sizeof(R) == 8 ? 8 : 36);
     static constexpr int KG = NV / RG;
     static constexpr int EH = 8 / (RG * RC);
     static constexpr int RT = NB * RC;
@@ -132,11 +132,18 @@ __global__ void __launch_bounds__(TT, 2) restrict_kernel(C<R> *__restrict__ cout
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
 
-    C<R> acc[KG][NB];
+    // FP32: the products of a piece are summed first, four roundings at their size
+    // and one at that of the running sum instead of four at that.  FP64 (one
+    // element per piece, bound by its pipe): the two products of a part in chains
+    // of their own, each rounding at a fraction of the sum.
+    constexpr int CH = EPP == 1 ? 2 : 1;
+    C<R> acc[KG][NB][CH];
 #pragma unroll
     for (int a = 0; a < KG; ++a)
 #pragma unroll
-        for (int r = 0; r < NB; ++r) acc[a][r] = mk<R>(0, 0);
+        for (int r = 0; r < NB; ++r)
+#pragma unroll
+            for (int h = 0; h < CH; ++h) acc[a][r][h] = mk<R>(0, 0);
 #pragma unroll
     for (int i = 0; i < NS - 1; ++i) fill(st0 + i);
     for (unsigned st = st0; st < st1; ++st) {
@@ -154,9 +161,20 @@ __global__ void __launch_bounds__(TT, 2) restrict_kernel(C<R> *__restrict__ cout
             C<R> v[EPP];
             unpiece(*reinterpret_cast<const typename P::FP *>(sf + r * SE), v);
 #pragma unroll
-            for (int a = 0; a < KG; ++a)
+            for (int a = 0; a < KG; ++a) {
+                if constexpr (CH == 2) {
+                    C<R> &s0 = acc[a][r][0], &s1 = acc[a][r][1];
+                    s0.x += q[a][0].x * v[0].x;
+                    s0.y += q[a][0].x * v[0].y;
+                    s1.x += q[a][0].y * v[0].y;
+                    s1.y -= q[a][0].y * v[0].x;
+                } else {
+                    C<R> t = mk<R>(0, 0);
 #pragma unroll
-                for (int x = 0; x < EPP; ++x) cfmac(acc[a][r], q[a][x], v[x]);
+                    for (int x = 0; x < EPP; ++x) cfmac(t, q[a][x], v[x]);
+                    acc[a][r][0] = acc[a][r][0] + t;
+                }
+            }
         }
     }
     asm volatile("cp.async.wait_all;\n" ::: "memory");
@@ -168,7 +186,7 @@ __global__ void __launch_bounds__(TT, 2) restrict_kernel(C<R> *__restrict__ cout
     for (int a = 0; a < KG; ++a)
 #pragma unroll
         for (int r = 0; r < NB; ++r) {
-            C<R> v = acc[a][r];
+            C<R> v = CH == 2 ? acc[a][r][0] + acc[a][r][CH - 1] : acc[a][r][0];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
@@ -231,20 +249,28 @@ __global__ void __launch_bounds__(TT, 2) prolong_kernel(C<R> *__restrict__ f, co
                 for (int x = 0; x < EPP; ++x) v[r][x] = mk<R>(0, 0);
         }
         constexpr int KU = NB >= 6 ? (NV % 4 == 0 ? 4 : 2) : NV % 8 == 0 ? 8 : NV % 6 == 0 ? 6 : NV;
+        constexpr int KS = KU % 4 == 0 ? 4 : 2;
 #pragma unroll 1
         for (int k0 = 0; k0 < NV; k0 += KU) {
             typename P::QP w[KU];
 #pragma unroll
             for (int k = 0; k < KU; ++k)
                 w[k] = *reinterpret_cast<const typename P::QP *>(Q + (int64_t)(k0 + k) * m.nelem + a);
+            // KS rows' products first, then the running sum: it rounds once per KS rows
 #pragma unroll
-            for (int k = 0; k < KU; ++k) {
-                C<R> q[EPP];
-                P::q(w[k], q);
+            for (int k = 0; k < KU; k += KS) {
+                C<R> q[KS][EPP];
+#pragma unroll
+                for (int j = 0; j < KS; ++j) P::q(w[k + j], q[j]);
 #pragma unroll
                 for (int r = 0; r < NB; ++r)
 #pragma unroll
-                    for (int x = 0; x < EPP; ++x) cfma(v[r][x], q[x], cs[k0 + k][r]);
+                    for (int x = 0; x < EPP; ++x) {
+                        C<R> t = mk<R>(0, 0);
+#pragma unroll
+                        for (int j = 0; j < KS; ++j) cfma(t, q[j][x], cs[k0 + k + j][r]);
+                        v[r][x] = v[r][x] + t;
+                    }
             }
         }
 #pragma unroll

@@ -120,3 +120,36 @@ def test_coarsest_gcr(G, dims, Ls, nvec, block, restart, its, f32, f64, prec):
         err += _rel(x, _gcr64(Y, d, b.to(torch.complex128), its, restart)) / 4
     assert err < 1.15 * (f32 * 1e-7 if prec else f64 * 1e-16)
     ctx.close()
+
+
+@pytest.mark.parametrize("dims,Ls,nvec,block,restrict,prolong",
+                         [((8, 8, 8, 8), 8, 8, (2, 2, 2, 2), 1.00, 0.63), ((8, 8, 8, 8), 4, 16, (2, 2, 2, 2), 0.95, 0.82),
+                          ((8, 8, 8, 8), 16, 24, (4, 4, 4, 4), 2.7, 0.98), ((6, 6, 4, 8), 12, 32, (3, 3, 2, 4), 1.49, 1.11)])
+def test_fp32_transfers(G, dims, Ls, nvec, block, restrict, prolong):
+    """One restriction and one prolongation against FP64 on the same basis: what
+    sums of whole products leave (1e-7), 4 % between inputs."""
+    ctx = _ctx(dims, Ls)
+    p = M._params(G, setup_iters0=4, setup_sweeps=0, smoother_prec=1, coarse_prec=[1])
+    G.mg_setup(ctx.h, 2, [nvec], [block], p, torch.from_numpy(I.random_vectors(nvec // 2, dims, Ls, 3)).cuda())
+    N = ctx.field_elems
+    Q = torch.empty(nvec * N, dtype=torch.complex128, device="cuda")
+    G.mg_get_vectors(ctx.h, 0, Q)
+    torch.cuda.synchronize()
+    Q = Q.reshape(nvec, N)
+    d, n = G.mg_level_info(ctx.h, 1)
+    site, xc, m = torch.arange(int(np.prod(dims)), device="cuda"), 0, 1
+    for mu in range(4):
+        xc = xc + (site % dims[mu] // block[mu]) * m
+        site, m = site // dims[mu], m * d[mu]
+    xc = xc.repeat_interleave(12 * Ls)  # the block of every element
+    err = np.zeros(2)
+    for s in range(4):
+        f, out = _randn(N, 5 + s, torch.complex64).to(torch.complex128), torch.empty(m * n, dtype=torch.complex128, device="cuda")
+        G.mg_restrict(ctx.h, 0, out, f)
+        ref = torch.zeros(n, m, dtype=torch.complex128, device="cuda").index_add_(1, xc, Q.conj() * f)
+        err[0] += _rel(out, ref.T.reshape(-1)) / 4
+        c, out = _randn(m * n, 50 + s, torch.complex64).to(torch.complex128), torch.empty(N, dtype=torch.complex128, device="cuda")
+        G.mg_prolong(ctx.h, 0, out, c)
+        err[1] += _rel(out, (Q * c.reshape(m, n).T[:, xc]).sum(0)) / 4
+    assert err[0] < 1.04e-7 * restrict and err[1] < 1.04e-7 * prolong
+    ctx.close()
