@@ -57,6 +57,21 @@ template <typename T> __host__ __device__ __forceinline__ void cfmac(T &acc, T a
     acc.y -= a.y * b.x;
 }
 
+// the same for long sums: s0 + s1 += a * b (conj(a) * b), the two products of a
+// part in chains of their own.  One chain of both rounds four times per product
+// at the size of the sum, two chains at a fraction of it.
+template <typename T> __host__ __device__ __forceinline__ void cfma2(T &s0, T &s1, T a, T b) {
+    s0.x += a.x * b.x;
+    s0.y += a.x * b.y;
+    s1.x -= a.y * b.y;
+    s1.y += a.y * b.x;
+}
+template <typename T> __host__ __device__ __forceinline__ void cfmac2(T &s0, T &s1, T a, T b) {
+    s0.x += a.x * b.x;
+    s0.y += a.x * b.y;
+    s1.x += a.y * b.y;
+    s1.y -= a.y * b.x;
+}
 // acc += a * b with the product formed on its own: six instructions, of which
 // one rounds at the size of acc where each of cfma's four does.  For vector
 // updates, whose products are small against what they are added to.

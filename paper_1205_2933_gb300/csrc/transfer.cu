@@ -163,11 +163,7 @@ __global__ void __launch_bounds__(TT, 2) restrict_kernel(C<R> *__restrict__ cout
 #pragma unroll
             for (int a = 0; a < KG; ++a) {
                 if constexpr (CH == 2) {
-                    C<R> &s0 = acc[a][r][0], &s1 = acc[a][r][1];
-                    s0.x += q[a][0].x * v[0].x;
-                    s0.y += q[a][0].x * v[0].y;
-                    s1.x += q[a][0].y * v[0].y;
-                    s1.y -= q[a][0].y * v[0].x;
+                    cfmac2(acc[a][r][0], acc[a][r][1], q[a][0], v[0]);
                 } else {
                     C<R> t = mk<R>(0, 0);
 #pragma unroll

@@ -153,3 +153,40 @@ def test_fp32_transfers(G, dims, Ls, nvec, block, restrict, prolong):
         err[1] += _rel(out, (Q * c.reshape(m, n).T[:, xc]).sum(0)) / 4
     assert err[0] < 1.04e-7 * restrict and err[1] < 1.04e-7 * prolong
     ctx.close()
+
+
+@pytest.mark.parametrize("dag", [False, True])
+@pytest.mark.parametrize("prec", [0, 1], ids=["f64", "f32"])
+@pytest.mark.parametrize("dims,Ls,nvec,block,f32,f64", [((8, 8, 8, 8), 8, 8, (2, 2, 2, 2), 2.12, 4.2),
+                                                        ((8, 8, 8, 8), 8, 24, (4, 4, 2, 2), 3.57, 6.9),
+                                                        ((8, 8, 8, 8), 4, 32, (2, 2, 2, 2), 4.11, 7.9)])
+def test_coarse_operator(G, dims, Ls, nvec, block, f32, f64, prec, dag):
+    """The coarse stencil, D and D^+, against FP64 on the same links: what one
+    chain of whole products over all 9 Nvec links leaves (f32 1e-7, f64 1e-16;
+    the latter with the reference's own)."""
+    ctx = _ctx(dims, Ls)
+    p = M._params(G, setup_iters0=4, setup_sweeps=0, smoother_prec=prec, coarse_prec=[prec])
+    G.mg_setup(ctx.h, 2, [nvec], [block], p, torch.from_numpy(I.random_vectors(nvec // 2, dims, Ls, 3)).cuda())
+    d, n = G.mg_level_info(ctx.h, 1)
+    V, dt = int(np.prod(d)), torch.complex64 if prec else torch.complex128
+    y = torch.empty(V * 9 * n * n, dtype=torch.complex128, device="cuda")
+    G.mg_get_coarse_links(ctx.h, 1, y)
+    Y = y.to(dt).to(torch.complex128).reshape(V, 9, n, n)
+    site = torch.arange(V, device="cuda").reshape(tuple(d)[::-1])
+    nb = [site.reshape(-1)]
+    for mu in range(4):
+        nb += [torch.roll(site, s, 3 - mu).reshape(-1) for s in (-1, 1)]
+    err = 0.0
+    for s in range(4):
+        b = _randn(V * n, 7 + s, dt)
+        out, v = torch.empty_like(b), b.to(torch.complex128).reshape(V, n)
+        G.mg_coarse_apply(ctx.h, 1, out, b, dagger=dag, prec=prec)
+        if dag:  # D^+ v at x: Y_d(y)^+ v(y) of the sites y whose direction d leads to x
+            ref = torch.zeros_like(v)
+            for k in range(9):
+                ref.index_add_(0, nb[k], torch.einsum("slk,sl->sk", Y[:, k].conj(), v))
+        else:
+            ref = sum(torch.einsum("skl,sl->sk", Y[:, k], v[nb[k]]) for k in range(9))
+        err += _rel(out, ref.reshape(-1)) / 4
+    assert err < 1.05 * (f32 * 1e-7 if prec else f64 * 1e-16)
+    ctx.close()
