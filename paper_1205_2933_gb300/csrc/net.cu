@@ -70,11 +70,11 @@ __global__ void __launch_bounds__(256) cgemm_kernel(float2 *__restrict__ C, cons
     const int m0 = blockIdx.y * GBM, n0 = blockIdx.x * GBN;
     const int kbeg = blockIdx.z * kchunk;
     const int kend = min(K, kbeg + kchunk);
-    float2 acc[4][4];
+    float2 acc[4][4], acc2[4][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+        for (int j = 0; j < 4; ++j) acc[i][j] = acc2[i][j] = make_float2(0.f, 0.f);
     for (int k0 = kbeg; k0 < kend; k0 += GBK) {
         for (int e = tid; e < GBK * GBM; e += 256) {
             int kk, mm;
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(256) cgemm_kernel(float2 *__restrict__ C, cons
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) cfma(acc[i][j], av[i], bv[j]);
+                for (int j = 0; j < 4; ++j) cfma2(acc[i][j], acc2[i][j], av[i], bv[j]);
         }
         __syncthreads();
     }
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(256) cgemm_kernel(float2 *__restrict__ C, cons
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int m = m0 + ty + 16 * i, n = n0 + tx + 16 * j;
-            if (m < M && n < N) Cz[(int64_t)m * N + n] = acc[i][j];
+            if (m < M && n < N) Cz[(int64_t)m * N + n] = acc[i][j] + acc2[i][j];
         }
 }
 
@@ -376,9 +376,10 @@ __global__ void __launch_bounds__(NT) block_gram_kernel(double2 *__restrict__ Gp
             const int p = threadIdx.x + q * NT;
             if (p < np) {
                 const int k = p / nf, l = p - k * nf;
-                float2 s = make_float2(0.f, 0.f);
+                float2 s = make_float2(0.f, 0.f), s1 = s;
 #pragma unroll 8
-                for (int e = 0; e < GCH; ++e) cfmac(s, sF[k * GCH + e], sF[l * GCH + e]);
+                for (int e = 0; e < GCH; ++e) cfmac2(s, s1, sF[k * GCH + e], sF[l * GCH + e]);
+                s = s + s1;
                 acc[q].x += (double)s.x;
                 acc[q].y += (double)s.y;
             }

@@ -190,3 +190,18 @@ def test_coarse_operator(G, dims, Ls, nvec, block, f32, f64, prec, dag):
         err += _rel(out, ref.reshape(-1)) / 4
     assert err < 1.05 * (f32 * 1e-7 if prec else f64 * 1e-16)
     ctx.close()
+
+
+def test_network_forward(G):
+    """The FP32 network (48 channels, three layers) against the FP64 oracle: 7.5e-7
+    with sums of whole products, a tenth more allowed."""
+    import test_gpu_net as T
+    from oracle import net as N
+    shape = N.NetShape(c_in=8, hidden=48, layers=3, nout=6, Ls=8)
+    U = I.epsilon_links(T.DIMS, 0.3, 1)
+    c = T.NetCase(G, U, shape)
+    h0 = T._input(shape, T.DIMS, 20)
+    ref, _ = N.forward(shape, c.p, U, h0, T.DIMS)
+    out = c.forward(h0=h0)
+    assert np.linalg.norm(out.reshape(-1) - ref.reshape(-1)) < 8.2e-7 * np.linalg.norm(ref)
+    c.close()
