@@ -616,10 +616,12 @@ template <typename R> class Runner {
 // rounds off z stays in it (FP32 V-cycle with 16 steps: 1.3e-7 against 3.7e-7 of
 // the result; 8 steps of the relaxation: 1.3e-6 against 3.2e-6 of the vectors).
 // The carried form serves FP32 batches at the extents that leave no lane of the
-// paired Dslash's warps idle (Ls / 2 divides 32): theirs is the rounding that
-// callers of several sources have always had there, and keeping r would cost
-// them a third of their time (V-cycle of 12 fields, 12^3 x 16 x 16). One
-// right-hand side, FP64 and the other extents keep r, as they always did.
+// paired Dslash's warps idle (Ls / 2 divides 32): it is the rounding that several
+// sources have always had there, and keeping r would cost them 45 % of a V-cycle
+// (12 fields, 12^3 x 16 x 16: 13.5 -> 19.5 ms) and 36 % of the relaxation (12
+// vectors, 600 steps, 16^3 x 32 x 16: 0.91 -> 1.25 s).  One right-hand side, FP64
+// and the other extents have always kept r, and a form that rounds worse is not
+// for them.
 bool carried_form(int Ls, int nr, bool f32) { return f32 && nr > 1 && Ls >= 4 && Ls % 2 == 0 && 32 % (Ls / 2) == 0; }
 
 // Batched solve: all right-hand sides advance together.  Fine-level kernels
