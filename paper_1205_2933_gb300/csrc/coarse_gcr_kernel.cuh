@@ -377,14 +377,15 @@ template <typename R, typename LT, int NV> __device__ __forceinline__ C<R> row_t
 // for the reduction.  The products <W_i, w>, |w|^2 and <w, r> are reduced
 // together: with W orthonormal |w|^2 loses sum |<W_i, w>|^2 in the projection
 // and <w, r> does not change (r is orthogonal to the W_i).  Where the
-// projection took 1 % or more of |w|^2, where that difference and the W_i's
+// projection took a tenth or more of |w|^2, where that difference and the W_i's
 // rounding would lose digits, a second one follows with a reduction of its own
-// (always taking two rounds no better).  The stencil: one
+// (at 3/4 FP64 rounds 1.1 times worse than with two projections each, at a
+// hundredth no better).  The stencil: one
 // thread per (direction, row) of a site, the neighbours' values staged.
 // Bound by the latency of the two barriers and of one L2 round trip after
-// each: 512 sites x 24 in BF16 44 us where the vectors in global memory, four
-// barriers per iteration and FP64 sums took 118; 256 sites x 16 in FP64 76 us
-// against 673.
+// each: 512 sites x 24 in BF16 52 us a call where the vectors in global memory,
+// four barriers per iteration and FP64 sums took 117; 256 sites x 16 in FP64 (a
+// V-cycle's) 0.09 ms against 0.67.
 template <typename R, typename LT, int NV, int NPTS>
 __global__ void __launch_bounds__(CT) coarse_gcr_smem_kernel(Args<R, LT> a, int spc, int cached) {
     using A = typename AccT<R>::type;
@@ -540,7 +541,7 @@ __global__ void __launch_bounds__(CT) coarse_gcr_smem_kernel(Args<R, LT> a, int 
                     z[e] = zv;
                 }
                 __syncthreads();  // tot is rewritten by the next reduction
-                const bool again = pass == 0 && removed >= 0.01 * ww;
+                const bool again = pass == 0 && removed >= 0.1 * ww;
                 ww -= removed;
                 if (!again) break;
             }

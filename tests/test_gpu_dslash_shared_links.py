@@ -80,3 +80,17 @@ def test_vcycle_field_by_field(G, dims, Ls, nrhs, rb, few):
         torch.cuda.synchronize()
         assert ((x[r] - y).norm() / y.norm()).item() < 1e-5, r
     ctx.close()
+
+
+@pytest.mark.parametrize("Ls", [4, 6, 10, 12, 16, 20, 24, 32, 48, 64])
+def test_carried_updates_of_cg(G, Ls):
+    """Eleven CG iterations, whose z and w the Dslash epilogues update, in FP32
+    against FP64 (3e-7 per eight iterations at Ls 8, thirty times that)."""
+    dims = (6, 4, 4, 6)
+    ctx = _ctx(dims, Ls)
+    b = torch.randn(ctx.field_elems, dtype=torch.complex128, device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+    x = [torch.zeros_like(b), torch.zeros_like(b)]
+    for i in (0, 1):
+        assert G.dwf_cg_solve(ctx.h, b, x[i], 1e-14, 11, 1, i, check=False).iters == 11
+    assert ((x[1] - x[0]).norm() / x[0].norm()).item() < 1e-5
+    ctx.close()
