@@ -109,10 +109,12 @@ typedef struct {
                                except along lattice directions of extent 1;
                                the V-cycle restricts D^+ r instead of r, and several right-hand
                                sides are solved one after another) (0) */
-    int graph;              /* 1: the batched V-cycle (FP32, two levels, several right-hand sides)
-                               is captured once per solve call, batch width and direction slot as a
-                               CUDA graph and replayed; 0: launched kernel by kernel.  Ignored for a
-                               lattice of a batch context (dwf_create with nlat > 1) (1) */
+    int graph;              /* 1: the solve's V-cycle (two levels, nu_pre = 0; FP32 for any number of
+                               right-hand sides, FP64 for one at a time) is captured once per solve
+                               call, batch width and direction slot as a CUDA graph and replayed;
+                               0: launched kernel by kernel, as it is with coarse_restart > 32 (whose
+                               coarsest solve reads its scalars on the host) and for a lattice of a
+                               batch context (dwf_create with nlat > 1) (1) */
 } mg_params;
 
 typedef struct {
@@ -350,13 +352,16 @@ void dwf_destroy(dwf_ctx *ctx);
  *   DWF_DSLASH_PAIR_MINB=4   paired FP32 Dslash in 128-thread CTAs, 4 per SM
  *                            (default: 64 threads, 8 per SM)
  *   DWF_DSLASH_MINB=6        one-slice Dslash at 80 registers, 6 CTAs per SM
- *   DWF_BATCH=0              several right-hand sides solved one at a time
+ *   DWF_BATCH=0              V-cycles of the launch-by-launch smoother, one
+ *                            right-hand side at a time (also where there is
+ *                            only one, and in FP64)
  *   DWF_COARSE_BATCH=0       the batched V-cycle's coarsest solves one
  *                            right-hand side per cooperative launch
- *   DWF_SMOOTHER_HISTORY=0   the CGNR smoother and setup relaxation with a
- *                            direction vector instead of the form that keeps
- *                            its residuals, and dwf_cg_solve one launch per
- *                            vector update (read at every solve call)
+ *   DWF_SMOOTHER_HISTORY=0   the CGNR smoother and setup relaxation with one
+ *                            direction vector and x updated as they go instead
+ *                            of keeping all directions or residuals, and
+ *                            dwf_cg_solve one launch per vector update (read
+ *                            at every solve call)
  *   DWF_TC_FORCE_WAIT=n      test hook: the first n launches of the
  *                            tensor-core coarsest solver begin with a wait
  *                            that runs out after about one second (the call

@@ -3,15 +3,18 @@
 //
 // The coarsest problem is small (e.g. 512 sites x 24 components) and a GCR
 // iteration built from separate launches is bound by launch and host
-// round-trip latency.  Here a co-resident grid (about one element per
-// thread, at most one CTA per SM) owns contiguous slices of every coarse
-// vector; grid-wide barriers separate the stencil apply (which reads
-// other slices) and the reductions.  Each reduction writes one FP64 partial
-// per CTA; after the barrier every CTA adds the partials in the same order,
-// so all CTAs hold bit-identical scalars and take identical loop decisions.
-// The algorithm is the same GCR as the launch-by-launch version: classical
-// Gram-Schmidt twice against the stored directions, |w| normalisation,
-// x += <w,r> z, r -= <w,r> w, true residual at each restart.
+// round-trip latency.  Here a co-resident grid (whole sites per CTA, at most
+// one CTA per SM) owns contiguous slices of every coarse vector, in shared
+// memory where they fit and else in global memory (coarse_gcr_kernel.cuh has
+// both kernels); grid-wide barriers separate the stencil apply (which reads
+// other slices) and the reductions.  Each reduction writes one partial per CTA
+// (FP64; pairs of FP32 numbers for FP32 fields in shared memory); after the
+// barrier every CTA adds the partials in the same order, so all CTAs hold
+// bit-identical scalars and take identical loop decisions.  The algorithm is
+// the GCR of the launch-by-launch version: classical Gram-Schmidt against the
+// stored directions, twice where the first pass took a tenth of |w|^2 or more
+// (in global memory always twice), |w| normalisation, x += <w,r> z,
+// r -= <w,r> w, true residual at each restart.
 #include <mutex>
 
 #include "coarse_gcr_kernel.cuh"

@@ -208,7 +208,7 @@ void launch(dwf_ctx *c, C<R> *out, const C<R> *in, const C<R> *U, bool dag, int 
     const bool shfl = (32 % g.Ls) == 0;
     // FP64: smaller CTAs while the grid has less than six of them per SM, so that
     // the FP64 pipes finish together (256 CTAs of 128 threads leave every third
-    // of 152 SMs' pipes idle half of the time: the FP64 V-cycle at 8^4 x 8 takes
+    // of 152 SMs' pipes idle half of the time: the FP64 V-cycle at 8^4 x 8 took
     // 1.58 ms with them, 1.50 with 1024 of 32)
     if (sizeof(R) == 8)
         while (spb > 1 && spb / 2 * g.Ls >= 32 && (g.V + spb - 1) / spb * nrhs < 6 * (int64_t)c->sm_count) spb /= 2;

@@ -1,5 +1,7 @@
-// FP32 fine Dslash with two fifth-dimension slices per thread (any even Ls up
-// to 64; each includer instantiates some of them).
+// FP32 fine Dslash with two fifth-dimension slices per thread, written for any
+// even Ls up to 64 and instantiated for 4, 6, 8, 10, 12, 16, 20, 24, 32, 48 and
+// 64 (each includer has some of them).  Every other Ls takes the one-slice kernel
+// of dslash.cu, slower and without these epilogues.
 //
 // Same operator as dslash.cu (Sec. 2: Shamir domain-wall operator; Sec. 4:
 // 11-site stencil).  A thread owns the slices s0 = 2j and s1 = 2j + 1 of one
@@ -126,8 +128,8 @@ __device__ __forceinline__ void recon2(CP acc[12], int a, const CP &u0, const CP
 
 // One 4D hop for both slices from the neighbour's preloaded row p (the 12
 // components of the thread's two slices).  sL: the staged link (9 elements
-// as float4 (re, re, im, im), hop coefficient included); ADJ: use its
-// adjoint.
+// (re, im), hop coefficient included; each part is duplicated in registers);
+// ADJ: use its adjoint.
 template <int MU, bool ADJ>
 __device__ __forceinline__ void hop2(CP acc[12], const float4 p[12], const float2 *sL, float sig) {
     float2 lk[10];
@@ -207,8 +209,8 @@ __device__ __forceinline__ void st_hint(float4 *p, const float4 &v, uint64_t pol
 // exceed L1, so 87 % of them are also filled whatever the shape of the CTA's
 // sites.  Hence: the links as 16-byte loads of two elements instead of one
 // element with both parts duplicated (443 -> 419 us), two right-hand sides per
-// staged link (four leave too few CTAs in small grids, 12 % slower at 5040 sites
-// x 3), and the second field of the fused kernels asked for by an L2 prefetch
+// staged link (from Ls 10 on four leave too few CTAs in small grids, 12 % slower
+// at 5040 sites x 3 x Ls 12; dslash_pair_ls has the rule), and the second field of the fused kernels asked for by an L2 prefetch
 // and loaded while the last hop computes, which leaves shared memory to L1 and
 // lets them share links as well (362 -> 333 us for 12 fields of 12^3 x 16 x 16
 // against staging it by cp.async).  The CTA's sites are a brick (Brick) so that
@@ -271,7 +273,7 @@ dslash_pair_kernel(float2 *out0, const float2 *in0, const float2 *__restrict__ U
     const int site = site_of(g, x);
     // the links of the CTA's sites: U_mu(x) and U_mu(x-mu), two stored rows, the
     // third rebuilt as conj(row0 x row1) (det U = 1), scaled by the hop
-    // coefficient and duplicated into (re, re, im, im)
+    // coefficient, (re, im) per element
     for (int jj = threadIdx.x; jj < spb * 8; jj += blockDim.x) {
         const int k = jj & 7, mu = k & 3;
         int y[4];

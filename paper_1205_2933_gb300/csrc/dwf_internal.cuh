@@ -126,8 +126,9 @@ void note_launches(unsigned long long n);  // kernels launched by a replayed gra
 // the kernel runs).  pdl_dependents comes
 // late in the kernels here: CTAs that start while the grid before still fills
 // most SMs settle unevenly on what is left, which a grid of one wave never
-// makes up (FP64 V-cycle at 8^4 x 8: 2.28 ms with the call first, 1.50 without
-// dependent launch, 1.43 with the call before the epilogue).
+// makes up (FP64 V-cycle at 8^4 x 8, when its epilogues carried z and w: 2.28 ms
+// with the call first, 1.50 without dependent launch, 1.43 with the call before
+// the epilogue).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -1514,10 +1514,10 @@ bool batch_on() {
 }
 
 // The batched path covers V-cycles on two levels with nu_1 = 0, one right-hand
-// side included (its smoother then needs 2 launches per step instead of 6: a
-// FP32 V-cycle at 8^3 x 16 x 16 in 1.07 ms instead of 1.50 when it moved here,
-// 0.77 now; an FP64 one at 8^4 x 8 in 1.43 ms instead of 1.65), FP64 always
-// one at a time.  An FP16 basis copy is used only by the other V-cycle.
+// side included (its smoother then needs 4 launches and 2 norm sums per step
+// instead of 8 launches: a FP32 V-cycle at 8^3 x 16 x 16 in 0.99 ms instead of
+// 2.4 before the transfers were cut into clusters, an FP64 one at 8^4 x 8 in
+// 1.52 ms instead of 2.9), FP64 always one at a time.  An FP16 basis copy is used only by the other V-cycle.
 // DWF_BATCH=0 in the environment turns it off.
 template <typename R> bool batch_eligible(const MGState &mg, int nrhs) {
     return (nrhs > 1 || !mg.lev[0].Q16.p) && batch_on() && mg.nlevels == 2 && mg.p.nu_pre == 0 &&

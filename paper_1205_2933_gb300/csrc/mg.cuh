@@ -104,7 +104,8 @@ void basis_to_half(dwf_ctx *c, __half2 *out, const float2 *in, int64_t n);
 template <typename R> void restrict_batch(dwf_ctx *c, const Level &L, C<R> *cout, const C<R> *fin, const C<R> *Q, int nrhs);
 template <typename R>
 void prolong_batch(dwf_ctx *c, const Level &L, C<R> *fout, const C<R> *cin, const C<R> *Q, int nrhs, bool accumulate);
-// G[Vc][nv][nv] = block inner products <A_k, B_l> over each block (FP64 accumulate)
+// G[Vc][nv][nv] = block inner products <A_k, B_l> over each block (FP64 fields: FP64 sums;
+// FP32 fields: a thread's sums as pairs of FP32 numbers, about 48 bits, the rest in FP64)
 template <typename R> void block_gram(dwf_ctx *c, const Level &L, double2 *G, const C<R> *A, const C<R> *B);
 // F[(Vc 8 + dd)][nv][nv] = <Q_k, H_l> over the face of each block in direction
 // mu (dir > 0: its last layer, dd = 2 mu; else the first, dd = 2 mu + 1), H

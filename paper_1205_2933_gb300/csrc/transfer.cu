@@ -84,9 +84,10 @@ template <typename R, typename QT, int NV, int NB, int RC> struct RShape {
 // asynchronous copies and the cluster's first CTA adds the parts in a fixed
 // order through distributed shared memory.  Bound: reading the basis once
 // (FP32, 12 right-hand sides: the FMA pipe comes close, 8 NV nrhs flops per
-// element); the loop is 12 shared loads of 16 bytes for 288 FMAs per lane at
-// Nvec 24.  12 right-hand sides, Nvec 24, Ls 16, 4^4 blocks:
-// 0.42 ms for 12^3 x 16 (1.5 GB read: 3.6 TB/s) against 1.37 ms with one CTA
+// element); the loop is 12 shared loads of 16 bytes for 288 FMAs and 72 additions
+// per lane at Nvec 24.  12 right-hand sides, Nvec 24, Ls 16, 4^4 blocks:
+// 0.45 ms for 12^3 x 16 (1.5 GB read: 3.3 TB/s; 0.41 without the additions, see
+// the sums below) against 1.37 ms with one CTA
 // per site and four right-hand sides and loads in the loop; one right-hand
 // side at 8^3 x 16 (32 sites) 54 us against 429 us
 template <typename R, typename QT, int NV, int NB, int RC>
@@ -212,8 +213,9 @@ __global__ void __launch_bounds__(TT, 2) restrict_kernel(C<R> *__restrict__ cout
 // thread owns EPP elements, keeps NB sums for each and streams over the basis
 // rows, whose loads do not depend on one another; the coefficients are
 // broadcast from shared memory, two right-hand sides per load.  Bound by
-// reading the basis and writing the fields: 0.35 ms for 12 right-hand sides,
-// Nvec 24, at 12^3 x 16 x 16 (0.70 ms with one CTA per site), 49 us for one at
+// reading the basis and writing the fields: 0.40 ms for 12 right-hand sides,
+// Nvec 24, at 12^3 x 16 x 16 (0.70 ms with one CTA per site; 0.35 with one chain of
+// multiply-adds per element, which rounds 1.3 times worse), 49 us for one at
 // 8^3 x 16 x 16 (608 us)
 template <typename R, typename QT, int NV, int NB>
 __global__ void __launch_bounds__(TT, 2) prolong_kernel(C<R> *__restrict__ f, const C<R> *__restrict__ cin,
